@@ -1,5 +1,6 @@
 // lbm_aux.cuh -- initial state and diagnostics kernels, generic over the precision
-// policy (lbm_prec.cuh).  Both evaluate in FP64 and (de)quantise at the store / load.
+// policy (lbm_prec.cuh).  The diagnostics evaluate in FP64, the initial state in FP64 or
+// double words; both (de)quantise at the load / store.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -8,52 +9,160 @@
 
 namespace lbm {
 
+// Arithmetic type of the initial state's equilibria: FP64 for the FP64 policy, double words
+// (48 bits, on the FP32 pipes) for every other one.
+template <class R>
+using init_t = typename std::conditional<std::is_same<R, double>::value, double, df64>::type;
+
+// A value of the initial state as the policy's arithmetic type (rounded once).
+template <class R, class I>
+__device__ __forceinline__ R init_value(I v)
+{
+    if constexpr (std::is_same<I, df64>::value && std::is_same<R, float>::value) return __fadd_rn(v.hi, v.lo);
+    else return (R)v;
+}
+
+// eq. H inverted for one cell (the map, and what follows from it), FP64: rho H, T, rho, c_p, psi.
+template <int N>
+__device__ __forceinline__ void init_macro(const KParams& P, const double (&phi)[N], double T_in, double& rhoH, double& T,
+                                           double& rho, double& cp, double& psi)
+{
+    const Mix<N> m = mixture_core<N>(P, phi);
+    rhoH = inverse_map<N>(P, m, T_in);
+    double fl;
+    enthalpy_map<N, true>(P, m, rhoH, fl, T);
+    const double fs = 1.0 - fl;
+    rho = fma(fs, m.rs, fl * m.rl);
+    cp = fma(fs, m.cs, fl * m.cl);
+    psi = fs * m.dr;
+}
+
+// The same in double words, for a cell whose phase the input temperature decides with margin
+// (returns false for any other: the FP64 form is then asked).  Above the liquidus the cell is
+// liquid whatever its latent heat; below the solidus it is solid where it holds
+// phase-changing material.  Either way the map returns the temperature it was given.  The
+// screen runs on FP32 values of the inputs; its margin of 1e-5 of the magnitudes is 25
+// times their rounding.
+template <int N>
+__device__ __forceinline__ bool init_macro_decided(const KParams& P, const df64 (&phi)[N], df64 T, df64& rhoH, df64& rho,
+                                                   df64& cp, df64& psi)
+{
+    const Coef<float>& C = P.f;
+    float rs = 0.0f, rl = 0.0f, cs = 0.0f, cl = 0.0f, Lv = 0.0f, La = 0.0f;
+#pragma unroll
+    for (int p = 0; p < N; ++p) {
+        rs = fmaf(phi[p].hi, C.rho_s[p], rs);
+        rl = fmaf(phi[p].hi, C.rho_l[p], rl);
+        cs = fmaf(phi[p].hi, C.cp_s[p], cs);
+        cl = fmaf(phi[p].hi, C.cp_l[p], cl);
+        Lv = fmaf(phi[p].hi, C.rhoL[p], Lv);
+        La = fmaf(fabsf(phi[p].hi), C.rhoL[p], La);
+    }
+    const float t = T.hi, tolT = 1e-5f * (fabsf(t) + fabsf(C.T_sol) + fabsf(C.T_liq)) + 1e-30f;
+    const Coef<df64>& X = P.x;
+    if (t > C.T_liq + tolT) {
+        const float rcl = rl * cl, As = rs * cs * C.T_sol, Al = fmaf(rcl, C.T_liq, Lv);
+        const float h = fmaf(rcl, t - C.T_liq, Al);
+        const float tol = 1e-5f * (fabsf(As) + fabsf(rcl * C.T_liq) + fabsf(rcl * t) + La) + 1e-30f;
+        if (!(rl > 1e-20f && cl > 1e-20f && h > As + tol)) return false;
+        rho = mix_sum<N, df64>(phi, X.rho_l);
+        cp = mix_sum<N, df64>(phi, X.cp_l);
+        rhoH = rfma(rho * cp, T, mix_sum<N, df64>(phi, X.rhoL));
+        psi = df64(0);
+        return true;
+    }
+    if (t < C.T_sol - tolT && Lv > 1e-5f * La + 1e-30f && rs > 1e-20f && cs > 1e-20f) {
+        rho = mix_sum<N, df64>(phi, X.rho_s);
+        cp = mix_sum<N, df64>(phi, X.cp_s);
+        rhoH = rho * cp * T;
+        psi = mix_sum<N, df64>(phi, X.drho);
+        return true;
+    }
+    return false;
+}
+
 // t = 0 (Section 3 equilibria, Section 2 eq. H inverted): from phi_p, T, u build
 // rho H, then f_l, T, rho, c_p by eq. H / eq. 2; populations at equilibrium with
 // p = 0; mdot' = Q' = 0, psi' = psi, (phi_p u)' = phi_p u.
+//
+// The inputs are FP64 fields.  With everything in FP64 (and each of the 9 (N + 2) values
+// converted on the same unit) the kernel was bound by the 2-lane FP64 pipe for every policy:
+// 1676 us at 2048^2, N = 2, FP16 storage, against 95 us for its bytes.  The policies that
+// store FP32 or less, and double words, now work in double words (an FP32 result is the
+// double word rounded once): 250 us there.  FP64 decides the cells that eq. H does not decide
+// by a margin.
+// Populations come in opposite pairs, whose even and odd parts in c_i . u are shared.
 template <int N, class Pr>
-__global__ void init_kernel(const KParams P, const double* __restrict__ phi_in, const double* __restrict__ T_in,
+__global__ void __launch_bounds__(256, 2) init_kernel(const KParams P, const double* __restrict__ phi_in, const double* __restrict__ T_in,
                             const double* __restrict__ ux_in, const double* __restrict__ uy_in,
                             void* __restrict__ pop_base, typename Pr::TA* __restrict__ aux)
 {
     using R = typename Pr::R;
     using TA = typename Pr::TA;
+    using I = init_t<R>;
+    using K = exact_t<I>;
     const long long S = P.S;
     const PopView<Pr> pop = pop_view<Pr>(P, pop_base);
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < S; c += (long long)gridDim.x * blockDim.x) {
-        double phi[N];
+        double phd[N];
 #pragma unroll
-        for (int p = 0; p < N; ++p) phi[p] = LBM_LD(P, phi_in, p * S + c, N * S, 40);
-        const double ux = ux_in ? LBM_LD(P, ux_in, c, S, 41) : 0.0, uy = uy_in ? LBM_LD(P, uy_in, c, S, 42) : 0.0;
-        const Mix<N> m = mixture_core<N>(P, phi);
-        const double rhoH = inverse_map<N>(P, m, LBM_LD(P, T_in, c, S, 43));
-        double fl, T;
-        enthalpy_map<N, true>(P, m, rhoH, fl, T);
-        const double fs = 1.0 - fl;
-        const double rho = fma(fs, m.rs, fl * m.rl);
-        const double cp = fma(fs, m.cs, fl * m.cl);
-        const double uu = ux * ux + uy * uy;
-        const double E = P.d.E_ref * T, Z = rho * cp * T;
+        for (int p = 0; p < N; ++p) phd[p] = LBM_LD(P, phi_in, p * S + c, N * S, 40);
+        const double T0 = LBM_LD(P, T_in, c, S, 43);
+        const I ux = ux_in ? I(LBM_LD(P, ux_in, c, S, 41)) : I(0.0), uy = uy_in ? I(LBM_LD(P, uy_in, c, S, 42)) : I(0.0);
+        I phi[N], rhoH, T = I(T0), rho, cp, psi;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const double cu = cx(i) * ux + cy(i) * uy;
-            const double si = wgt(i) * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
-            st_pop<Pr, KIND_F>(P, pop, 0, i, c, (R)(rho * si), 44);
-            double he;
-            if (i == 0) he = rhoH - E + wgt(0) * (E - 1.5 * Z * uu);
-            else he = wgt(i) * (E + Z * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu));
-            st_pop<Pr, KIND_H>(P, pop, N + 1, i, c, (R)he, 45);
+        for (int p = 0; p < N; ++p) phi[p] = I(phd[p]);
+        bool decided = false;
+        if constexpr (!std::is_same<I, double>::value) decided = init_macro_decided<N>(P, phi, T, rhoH, rho, cp, psi);
+        if (!decided) {
+            double rH, Tm, r, cpd, ps;
+            init_macro<N>(P, phd, T0, rH, Tm, r, cpd, ps);
+            rhoH = I(rH);
+            T = I(Tm);
+            rho = I(r);
+            cp = I(cpd);
+            psi = I(ps);
+        }
+        const I E = coef<I>(P).E_ref * T, Z = rho * cp * T;
+        const I uu15 = K(1.5) * rfma(ux, ux, uy * uy);
+        auto put = [&](auto kind, int s, int i, I v) {
+            st_pop<Pr, decltype(kind)::value>(P, pop, s, i, c, init_value<R>(v), 44);
+        };
+        using F = std::integral_constant<int, KIND_F>;
+        using G = std::integral_constant<int, KIND_G>;
+        using H = std::integral_constant<int, KIND_H>;
+        const I w0 = wgt_r<I>(0);
+        put(F{}, 0, 0, -(w0 * rho * uu15));
+        put(H{}, N + 1, 0, (rhoH - E) + w0 * (E - Z * uu15));
 #pragma unroll
-            for (int p = 0; p < N; ++p)
-                st_pop<Pr, KIND_G>(P, pop, 1 + p, i, c, (R)(wgt(i) * phi[p] * (1.0 + 3.0 * cu)), 46);
+        for (int p = 0; p < N; ++p) put(G{}, 1 + p, 0, w0 * phi[p]);
+        // opposite pairs (1, 3), (2, 4), (5, 7), (6, 8)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = k < 2 ? 1 + k : 3 + k, j = opp(i);
+            const I w = wgt_r<I>(i);
+            const I cu = i == 1 ? ux : i == 2 ? uy : i == 5 ? ux + uy : uy - ux;
+            const I odd = K(3) * cu, even = rfma(K(4.5) * cu, cu, -uu15);
+            const I sp = even + odd, sm = even - odd;
+            const I wr = w * rho, wE = w * E, wZ = w * Z;
+            put(F{}, 0, i, wr * sp);
+            put(F{}, 0, j, wr * sm);
+            put(H{}, N + 1, i, rfma(wZ, sp, wE));
+            put(H{}, N + 1, j, rfma(wZ, sm, wE));
+#pragma unroll
+            for (int p = 0; p < N; ++p) {
+                const I wp = w * phi[p];
+                put(G{}, 1 + p, i, rfma(wp, odd, wp));
+                put(G{}, 1 + p, j, rfma(-wp, odd, wp));
+            }
         }
         LBM_ST(P, aux, aux_mdot() * S + c, P.aux_elems, 47, (TA)0.0);
         LBM_ST(P, aux, aux_Q() * S + c, P.aux_elems, 47, (TA)0.0);
-        LBM_ST(P, aux, aux_psi() * S + c, P.aux_elems, 47, (TA)(fs * m.dr));
+        LBM_ST(P, aux, aux_psi() * S + c, P.aux_elems, 47, (TA)init_value<R>(psi));
 #pragma unroll
         for (int p = 0; p < N; ++p) {
-            LBM_ST(P, aux, aux_phiux(p) * S + c, P.aux_elems, 48, (TA)(phi[p] * ux));
-            LBM_ST(P, aux, aux_phiuy(N, p) * S + c, P.aux_elems, 48, (TA)(phi[p] * uy));
+            LBM_ST(P, aux, aux_phiux(p) * S + c, P.aux_elems, 48, (TA)init_value<R>(phi[p] * ux));
+            LBM_ST(P, aux, aux_phiuy(N, p) * S + c, P.aux_elems, 48, (TA)init_value<R>(phi[p] * uy));
         }
     }
 }
