@@ -177,11 +177,11 @@ __global__ void mac_kernel(const KParams P, const double* __restrict__ pin, cons
     const PopView<PrecFP64> pv = pop_view<PrecFP64>(P, pin);
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < P.S;
          c += (long long)gridDim.x * blockDim.x) {
-        double ph[N], r, ps;
+        d1 ph[N], r, ps;
         halo_moments<N, PrecFP64>(P, pv, ain, c, ph, r, ps);
-        for (int p = 0; p < N; ++p) mac[p * P.S + c] = ph[p];
-        mac[N * P.S + c] = r;
-        mac[(N + 1) * P.S + c] = ps;
+        for (int p = 0; p < N; ++p) mac[p * P.S + c] = ph[p].v;
+        mac[N * P.S + c] = r.v;
+        mac[(N + 1) * P.S + c] = ps.v;
     }
 }
 

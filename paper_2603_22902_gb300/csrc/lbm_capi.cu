@@ -254,6 +254,8 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
             const double sig = num->sigma[p * LBM_MAXN + q];
             P.d.b2[p][q] = 2.0 * 3.0 / num->eps * sig;      // 2 beta_pq
             P.d.kk[p][q] = 3.0 * num->eps / 4.0 * sig;      // -k_pq
+            P.d.b4[p][q] = 2.0 * P.d.b2[p][q];
+            P.d.kk6[p][q] = P.d.kk[p][q] / 6.0;
             for (int s = 0; s < 4; ++s)
                 P.d.wet[s][p][q] = bc->kind[s] == LBM_BC_WALL ? 4.0 / num->eps * bc->wet_cos[s][p * LBM_MAXN + q] : 0.0;
         }
@@ -272,6 +274,12 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
     const double tau_g = num->mobility * 3.0 + 0.5;
     P.d.omega_g = 1.0 / tau_g;
     P.d.kg = 1.0 - 0.5 * P.d.omega_g;
+    P.d.omega_g1 = 1.0 - P.d.omega_g;
+    const double gc[5] = {3.0 * (P.d.omega_g + P.d.kg), -3.0 * P.d.kg, P.d.kg, P.d.omega_g, P.d.kg};
+    for (int k = 0; k < 5; ++k) P.d.g_sc[k] = gc[k];
+    for (int k = 0; k < 3; ++k) P.d.g_pl[k] = gc[k] / 9.0;
+    P.d.E_ref49 = 4.0 / 9.0 * P.d.E_ref;
+    P.ordered = th->T_sol <= 0.0 && th->T_liq >= 0.0 ? 1 : 0;
 
     const size_t pb = plane_bytes(h);
     P.rest_elems = (long long)(N + 2) * P.S;
@@ -280,6 +288,10 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
     P.d.inv_E_ref = 1.0 / P.d.E_ref;
     P.f = round_coef(P.d);
     P.x = split_coef(P.d);
+    // 1 - omega_g from each type's own omega_g: the collision keeps sum_i g_i only if the two add
+    // up to 1 in the type it runs in
+    P.f.omega_g1 = 1.0f - P.f.omega_g;
+    P.x.omega_g1 = df64(1.0 - (double)P.x.omega_g);
     P.dbg = nullptr;
     dispatch(N, h->precision, [&](auto n, auto pr) {
         using Pr = decltype(pr);

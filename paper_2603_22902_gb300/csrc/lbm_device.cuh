@@ -7,6 +7,7 @@
 
 #include "lbm_df64.cuh"
 #include "lbm_lattice.cuh"
+#include "lbm_vals.cuh"
 
 namespace lbm {
 
@@ -28,17 +29,6 @@ __host__ __device__ inline int tile_rows_count(int ty, const TileRows& r)
     return r.part == ROWS_INNER ? r.hi - r.lo : r.part == ROWS_EDGE ? ty - (r.hi - r.lo) : ty;
 }
 
-// Arithmetic helpers for the compute type R of a precision policy.
-__device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float rfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double rrsqrt(double a) { return rsqrt(a); }
-__device__ __forceinline__ float rrsqrt(float a) { return rsqrtf(a); }
-// Type of a constant that FP32 holds exactly (2, 3, 0.5, 4.5, ...) in arithmetic of
-// type R: R itself, except float for double words (a product with a float costs 5 FP32
-// instructions instead of 8).  FP64 arithmetic is unchanged by it.
-template <class R>
-using exact_t = typename std::conditional<std::is_same<R, df64>::value, float, R>::type;
-
 // Per-run coefficients used by the arithmetic of the step, in type T.  The host fills
 // a double, a float and a double-word copy, so a policy computing in FP32 or in
 // double-word arithmetic reads its own constants and converts nothing per cell
@@ -52,6 +42,7 @@ struct Coef {
     T pcm[MAXN];                  // 1 where L_p > 0 (the phase changes phase), else 0
     // Section 2 free energy: 2 beta_pq = 6 sigma_pq / eps and -k_pq = 3 eps sigma_pq / 4
     T b2[MAXN][MAXN], kk[MAXN][MAXN];
+    T b4[MAXN][MAXN], kk6[MAXN][MAXN];   // 2 b2 and kk / 6 (with g' / 2 and 6 lap)
     T four_eps;                   // 4 / eps
     T wet[4][MAXN][MAXN];         // (4 / eps) cos(theta_pq) per wall side (0 elsewhere)
     T E_ref;                      // rho_ref c_p,ref
@@ -59,6 +50,11 @@ struct Coef {
     T tau_h_scale;                // 1 / (rho_ref c_p,ref c_s^2)
     T us[2], accel[2];
     T omega_g, kg;                // 1 / tau_g and 1 - 1/(2 tau_g), tau_g = M / c_s^2 + 1/2
+    T omega_g1;                   // 1 - 1 / tau_g
+    // phase-field collision: 3 (omega_g + k_g), -3 k_g, k_g over 9 for plain populations (g_pl);
+    // as they are for populations divided by their weights, with omega_g, k_g (g_sc)
+    T g_pl[3], g_sc[5];
+    T E_ref49;                    // 4/9 rho_ref c_p,ref
     T Tw[4];                      // Dirichlet wall temperature
     T rhoL[MAXN];                 // rho_l^p L_p (the FP64 map reads KParams::rhoL)
     T T_sol, T_liq;               // (the FP64 map reads KParams::T_sol, T_liq)
@@ -69,6 +65,7 @@ struct Coef {
 struct KParams {
     int nx, ny, N;
     long long S;                  // plane stride in elements (nx * ny)
+    int ordered;                  // 1: T_sol <= 0 <= T_liq, so As <= Al - Lv in eq. H
     int bc[4], tbc[4];            // side kinds, sides 0 x-min, 1 x-max, 2 y-min, 3 y-max
     Coef<double> d;               // coefficients, FP64
     Coef<float> f;                // the same, rounded to FP32

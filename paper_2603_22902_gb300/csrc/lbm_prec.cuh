@@ -15,9 +15,8 @@
 //                                         density ratio of 100 turned into 1 % of rho and of T)
 //   h_i  -> h_i / (w_i rho_ref c_p,ref)  (= T + O(u) away from walls)
 // Lagged planes are stored as TA.  Arithmetic of the collision runs in R; the
-// liquid fraction always comes from the FP64 enthalpy map (eq. H); policies that compute
-// in FP32 or double words screen the cell first and run the FP64 map only where the
-// screen cannot decide f_l (map_cell in lbm_step.cuh).
+// liquid fraction is always the FP64 enthalpy map's (eq. H): an FP32 screen decides the cells that
+// are clearly liquid or solid, the others run the FP64 map (liquid_fraction in lbm_cell.cuh).
 //
 // NGUARD: the pairwise normal n_pq = grad phi_pq / |grad phi_pq| is set to zero where
 // |grad phi_pq| is below NGUARD times its own scale (phi_q |grad phi_p| + phi_p |grad phi_q|),
@@ -44,6 +43,9 @@
 namespace lbm {
 
 constexpr float F_SCALE = 1.0f / 4096.0f;
+
+// Species kinds of the moving planes (their 16-bit encodings differ).
+constexpr int KIND_F = 0, KIND_G = 1, KIND_H = 2;
 
 struct PrecFP64 {
     using R = double;
