@@ -191,8 +191,9 @@ int lbm_debug_bounds(lbm_handle* h, long long* out3);
 
 /* Tile shape (bx, by) of the fused step kernel; 0, 0 restores the default (32x8).  The
  * shape must be one of the compiled variants, 32x8, 32x4, 64x4 or 16x16, and 32x8 for
- * an LBM_DF64 handle (LBM_EINVAL otherwise).  Results of different shapes agree to
- * rounding, not bit for bit (each shape is compiled on its own). */
+ * an LBM_DF64 handle (LBM_EINVAL otherwise).  With no shape asked for, an LBM_FP64 handle
+ * whose lattice fills the GPU badly with 32x8 tiles uses smaller ones.  Every operation is
+ * rounded as written, so results do not depend on the shape. */
 int lbm_set_tile(lbm_handle* h, int bx, int by);
 
 

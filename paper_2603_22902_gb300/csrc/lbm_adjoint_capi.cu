@@ -172,7 +172,7 @@ extern "C" int lbm_adjoint_fl_loss(lbm_handle* h, const double* phi0, const doub
         }
         e = dispatch(N, LBM_FP64, [&](auto nn, auto pr) {
             return launch_step<decltype(nn)::value, decltype(pr)>(P, h->pop[a], h->pop[b], h->aux[a], h->aux[b],
-                                                                  h->tile, st);
+                                                                  lbm_step_tile(h), st);
         });
         if (e != cudaSuccess) return acuda(h, e, "step kernel");
         h->cur = b;
@@ -207,7 +207,7 @@ extern "C" int lbm_adjoint_fl_loss(lbm_handle* h, const double* phi0, const doub
             char* sbn = seg.as<char>() + (size_t)j * set_bytes;
             e = dispatch(N, LBM_FP64, [&](auto nn, auto pr) {
                 return launch_step<decltype(nn)::value, decltype(pr)>(P, pop_of(sa), pop_of(sbn), aux_of(sa), aux_of(sbn),
-                                                                      h->tile, st);
+                                                                      lbm_step_tile(h), st);
             });
             if (e != cudaSuccess) return acuda(h, e, "recompute step kernel");
         }

@@ -127,6 +127,31 @@ batch_step_kernel(const BatchTable T, int s)
                                    (TA*)C.aux[a ^ 1], ExportPtrs{}, local % C.tiles_x, local / C.tiles_x, smem);
 }
 
+// Per-step form of small FP64 groups: each tile of the list as eight tiles of 8x4, one warp
+// each (see fp64_small_tiles for the rule).  Five small cases, 69 tiles: one tile of 8 warps
+// keeps its SM's FP64 unit busy for 46 us while 83 SMs idle.
+template <int N, int TX, int TY, class Pr>
+__global__ void __launch_bounds__(BATCH_NT / BATCH_SUB, LBM_OCC(Pr) * BATCH_SUB / BATCH_NT)
+batch_substep_kernel(const BatchTable T, int s)
+{
+    static_assert(TX * TY == BATCH_NT && TX % 8 == 0 && TY % 4 == 0, "eight 8x4 tiles");
+    using TA = typename Pr::TA;
+    __shared__ KParams sP;
+    __shared__ typename Pr::R smem[tile_smem_elems<N, 8, 4, Pr>()];
+    const int t = blockIdx.x / BATCH_SUB, sub = blockIdx.x % BATCH_SUB;
+    const int c = __ldg(T.tile_case + t);
+    const BatchCase& C = T.cases[c];
+    const int local = t - C.first_tile;
+    const int bx = local % C.tiles_x * (TX / 8) + sub % (TX / 8), by = local / C.tiles_x * (TY / 4) + sub / (TX / 8);
+    const KParams& G = T.params[c];
+    if (bx * 8 >= G.nx || by * 4 >= G.ny) return;   // wholly beyond the lattice
+    load_params(sP, T.params + c);
+    __syncthreads();
+    const int a = (*(volatile unsigned char*)T.parity) ^ (s & 1);
+    step_tile<N, 8, 4, true, Pr>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
+                                 (TA*)C.aux[a ^ 1], ExportPtrs{}, bx, by, smem);
+}
+
 // Staged form: one block per tile of the flat list (32x8 tiles), step s of the call;
 // maps[2 c + k] are the tensor maps of case c's population and lagged set k.
 template <int N, class Pr>

@@ -57,7 +57,7 @@ struct lbm_batch {
     std::vector<BatchCase> cases;
     std::vector<int> group;                 // group (tile kind) of each case
     int group_tiles[NKIND] = {0, 0, 0}, group_first[NKIND] = {0, 0, 0};
-    long long group_cells[NKIND] = {0, 0, 0};
+    long long group_cells[NKIND] = {0, 0, 0}, group_subtiles[NKIND] = {0, 0, 0};
     unsigned char parity[NKIND] = {0, 0, 0};
     BatchCase* d_cases = nullptr;
     KParams* d_params = nullptr;
@@ -142,6 +142,7 @@ static int build_tables(lbm_batch* b)
     for (int g = 0; g < NKIND; ++g) {
         b->group_tiles[g] = 0;
         b->group_cells[g] = 0;
+        b->group_subtiles[g] = 0;
     }
     for (int c = 0; c < nc; ++c) {
         const lbm_handle* h = b->h[c];
@@ -158,6 +159,7 @@ static int build_tables(lbm_batch* b)
         for (long long k = 0; k < n; ++k) tiles[g].push_back(c);
         b->group_tiles[g] += (int)n;
         b->group_cells[g] += (long long)h->nx * h->ny;
+        b->group_subtiles[g] += (long long)((h->nx + 7) / 8) * ((h->ny + 3) / 4);
         const int p = b->parity[g];
         C.pop[p] = h->pop[h->cur];
         C.pop[p ^ 1] = h->pop[h->cur ^ 1];
@@ -194,6 +196,8 @@ static BatchTable group_table(const lbm_batch* b, int g)
 {
     BatchTable T{};
     T.total_tiles = b->group_tiles[g];
+    T.total_subtiles = b->group_subtiles[g];
+    T.sms = b->sms;
     T.cases = b->d_cases;
     T.params = b->d_params;
     T.tile_case = b->d_tile_case + b->group_first[g];

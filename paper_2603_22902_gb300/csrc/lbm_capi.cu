@@ -216,6 +216,7 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
     lbm_handle* h = new (std::nothrow) lbm_handle();
     if (!h) return fail(nullptr, LBM_ENOMEM, "host allocation failed");
     cudaError_t e = cudaGetDevice(&h->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e != cudaSuccess) {
         delete h;
         return fail(nullptr, LBM_ECUDA, std::string("no CUDA device: ") + cudaGetErrorString(e));
@@ -337,6 +338,7 @@ int lbm_set_tile(lbm_handle* h, int bx, int by)
     if (!h) return fail(nullptr, LBM_EINVAL, "NULL handle");
     if (bx == 0 && by == 0) {
         h->tile = TILE_32x8;
+        h->tile_auto = true;
         return LBM_OK;
     }
     for (int id = 0; id < TILE_COUNT; ++id) {
@@ -347,6 +349,7 @@ int lbm_set_tile(lbm_handle* h, int bx, int by)
                 return fail(h, LBM_EINVAL, "the LBM_DF64 policy is compiled for the 32x8 tile only");
             if (id != TILE_32x8) h->staged = false;  // the staged step is compiled for 32x8
             h->tile = id;
+            h->tile_auto = false;
             return LBM_OK;
         }
     }
@@ -442,7 +445,7 @@ int lbm_step(lbm_handle* h, long nsteps)
                                                                        h->aux[a], h->aux[b], h->stage_status,
                                                                        h->stream);
             return launch_step<decltype(n)::value, decltype(pr)>(h->P, h->pop[a], h->pop[b], h->aux[a], h->aux[b],
-                                                                 h->tile, h->stream);
+                                                                 lbm_step_tile(h), h->stream);
         });
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
         h->cur = b;
@@ -479,7 +482,8 @@ int lbm_get_fields(lbm_handle* h, double* phi, double* T, double* H, double* fl,
     }
     cudaError_t e = dispatch(h->N, h->precision, [&](auto n, auto pr) {
         return launch_export<decltype(n)::value, decltype(pr)>(h->P, h->pop[h->cur], h->aux[h->cur], dev[0], dev[1],
-                                                               dev[2], dev[3], dev[4], dev[5], dev[6], h->stream);
+                                                               dev[2], dev[3], dev[4], dev[5], dev[6], lbm_step_tile(h),
+                                                               h->stream);
     });
     if (e != cudaSuccess) return cuda_fail(h, e, "export kernel");
     if (where == LBM_HOST) {

@@ -15,6 +15,8 @@ struct lbm_handle {
     int precision = LBM_FP64;
     int diag_every = 0;
     int tile = lbm::TILE_32x8;
+    bool tile_auto = true;                // no shape asked for: FP64 takes its own (fp64_tile)
+    int sms = 0;
     lbm::KParams P{};
     void* pop[2] = {nullptr, nullptr};    // one population set each (rest + moving block)
     void* aux[2] = {nullptr, nullptr};    // 3 + 2N lagged planes each
@@ -38,6 +40,12 @@ struct lbm_handle {
     bool slab_inner_pending = false;      // lbm_slab_step_part: inner rows stepped, edge rows not yet
     std::string err;
 };
+
+// Tile shape of the handle's one-launch step.
+inline int lbm_step_tile(const lbm_handle* h)
+{
+    return h->tile_auto && h->precision == LBM_FP64 ? lbm::fp64_tile(h->nx, h->ny, h->sms) : h->tile;
+}
 
 // The six tensor maps of the staged step (boxes A..F of lbm_staged.cuh) over a population
 // set `pop` and a lagged set `aux` laid out like the handle's (16-bit storage, N = 2,

@@ -41,6 +41,10 @@ static cudaError_t launch_fused(const KParams& P, const void* pin, void* pout, c
             case TILE_32x4: return launch_fused_t<N, 32, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
             case TILE_64x4: return launch_fused_t<N, 64, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
             case TILE_16x16: return launch_fused_t<N, 16, 16, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
+            case TILE_8x4:
+                if constexpr (std::is_same<Pr, PrecFP64>::value)
+                    return launch_fused_t<N, 8, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
+                else return cudaErrorNotSupported;
             default: return launch_fused_t<N, 32, 8, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
         }
     }
@@ -55,10 +59,10 @@ cudaError_t launch_step(const KParams& P, const void* pin, void* pout, const voi
 
 template <int N, class Pr>
 cudaError_t launch_export(const KParams& P, const void* pin, const void* ain, double* phi, double* T, double* H,
-                          double* fl, double* ux, double* uy, double* p, cudaStream_t st)
+                          double* fl, double* ux, double* uy, double* p, int tile, cudaStream_t st)
 {
-    return launch_fused<N, false, Pr>(P, pin, nullptr, ain, nullptr, ExportPtrs{phi, T, H, fl, ux, uy, p}, TILE_32x8,
-                                      st);
+    return launch_fused<N, false, Pr>(P, pin, nullptr, ain, nullptr, ExportPtrs{phi, T, H, fl, ux, uy, p},
+                                      tile == TILE_8x4 ? TILE_8x4 : TILE_32x8, st);
 }
 
 template <int N, class Pr>
@@ -86,9 +90,12 @@ template <int N, class Pr>
 cudaError_t launch_init(const KParams& P, const double* phi, const double* T, const double* ux, const double* uy,
                         void* pop, void* aux, cudaStream_t st)
 {
-    long long blocks = (P.S + 255) / 256;
+    // blocks of two warps where the lattice would leave SMs without one of eight (FP64, film
+    // 16x256: 16 blocks and 16 us against 64 blocks and 6 us)
+    const int nt = P.S < 256 * 304 ? 64 : 256;
+    long long blocks = (P.S + nt - 1) / nt;
     if (blocks > 65535) blocks = 65535;
-    init_kernel<N, Pr><<<(int)blocks, 256, 0, st>>>(P, phi, T, ux, uy, pop, (typename Pr::TA*)aux);
+    init_kernel<N, Pr><<<(int)blocks, nt, 0, st>>>(P, phi, T, ux, uy, pop, (typename Pr::TA*)aux);
     return cudaGetLastError();
 }
 
@@ -150,20 +157,31 @@ cudaError_t batch_blocks_per_sm(int kind, int* out)
     }
 }
 
+template <int N, int TX, int TY, class Pr>
+static cudaError_t launch_batch_step_t(const BatchTable& T, int s, cudaStream_t st)
+{
+    if constexpr (std::is_same<Pr, PrecFP64>::value) {
+        if (fp64_small_tiles(T.total_tiles, T.total_subtiles, T.sms)) {
+            batch_substep_kernel<N, TX, TY, Pr><<<T.total_tiles * BATCH_SUB, BATCH_NT / BATCH_SUB, 0, st>>>(T, s);
+            return cudaGetLastError();
+        }
+    }
+    batch_step_kernel<N, TX, TY, Pr><<<T.total_tiles, BATCH_NT, 0, st>>>(T, s);
+    return cudaGetLastError();
+}
+
 template <int N, class Pr>
 cudaError_t launch_batch_step(const BatchTable& T, int kind, int s, cudaStream_t st)
 {
     if constexpr (single_shape<Pr>()) {
         if (kind != TILE_32x8) return cudaErrorNotSupported;
-        batch_step_kernel<N, 32, 8, Pr><<<T.total_tiles, BATCH_NT, 0, st>>>(T, s);
-        return cudaGetLastError();
+        return launch_batch_step_t<N, 32, 8, Pr>(T, s, st);
     } else {
         switch (kind) {
-            case TILE_64x4: batch_step_kernel<N, 64, 4, Pr><<<T.total_tiles, BATCH_NT, 0, st>>>(T, s); break;
-            case TILE_16x16: batch_step_kernel<N, 16, 16, Pr><<<T.total_tiles, BATCH_NT, 0, st>>>(T, s); break;
-            default: batch_step_kernel<N, 32, 8, Pr><<<T.total_tiles, BATCH_NT, 0, st>>>(T, s); break;
+            case TILE_64x4: return launch_batch_step_t<N, 64, 4, Pr>(T, s, st);
+            case TILE_16x16: return launch_batch_step_t<N, 16, 16, Pr>(T, s, st);
+            default: return launch_batch_step_t<N, 32, 8, Pr>(T, s, st);
         }
-        return cudaGetLastError();
     }
 }
 
@@ -228,7 +246,7 @@ cudaError_t launch_adj_init(const KParams& P, const double* phi0, const double* 
     template cudaError_t launch_staged<N, PR>(const KParams&, const StageMaps&, const void*, void*, const void*,   \
                                               void*, int*, cudaStream_t, TileRows);                                 \
     template cudaError_t launch_export<N, PR>(const KParams&, const void*, const void*, double*, double*, double*, \
-                                              double*, double*, double*, double*, cudaStream_t);                    \
+                                              double*, double*, double*, double*, int, cudaStream_t);               \
     template cudaError_t launch_init<N, PR>(const KParams&, const double*, const double*, const double*,           \
                                             const double*, void*, void*, cudaStream_t);                             \
     template cudaError_t launch_diag<N, PR>(const KParams&, const void*, const void*, double*, double*, cudaStream_t, \

@@ -13,7 +13,8 @@
 namespace lbm {
 
 // Compiled tile shapes of the fused step kernel (TX x TY threads, one cell each).
-enum TileId { TILE_32x8 = 0, TILE_32x4 = 1, TILE_64x4 = 2, TILE_16x16 = 3, TILE_COUNT = 4 };
+// TILE_8x4, one warp, is FP64's for small lattices and not among the shapes a caller can ask for.
+enum TileId { TILE_32x8 = 0, TILE_32x4 = 1, TILE_64x4 = 2, TILE_16x16 = 3, TILE_COUNT = 4, TILE_8x4 = 4 };
 inline bool tile_dims(int id, int& tx, int& ty)
 {
     switch (id) {
@@ -21,8 +22,28 @@ inline bool tile_dims(int id, int& tx, int& ty)
         case TILE_32x4: tx = 32; ty = 4; return true;
         case TILE_64x4: tx = 64; ty = 4; return true;
         case TILE_16x16: tx = 16; ty = 16; return true;
+        case TILE_8x4: tx = 8; ty = 4; return true;
         default: return false;
     }
+}
+
+// Whether an FP64 step over `tiles` tiles of 256 cells (32x8, 64x4, 16x16), which `subtiles` tiles of
+// 8x4 cover as well, should use the latter.  The step is bound by the SM's 2-lane FP64 unit, which
+// a warp instruction holds for 16 cycles, so its time is the warp-passes on the fullest SM: a
+// cell's update takes about six times the instructions of a ring position's moments, and a tile
+// of 8 warps has 3 warps of ring positions, a tile of one warp one.  The small tiles cost a tenth
+// more where every SM is full and win where the large ones leave SMs idle or unevenly filled.
+// Measured, us per step, 8x4 against 32x8 (N = 2): 16 x 256 26.1 / 39.8, 128^2 28.6 / 38.0, 192^2
+// 41.1 / 38.6, 256^2 57.4 / 59.5, 384^2 117.5 / 114.5, 448^2 160 / 166, 512^2 201 / 193; the rule takes
+// the faster one at each of these, and for N = 3 and 4.
+inline bool fp64_small_tiles(long long tiles, long long subtiles, int sms)
+{
+    return (subtiles + sms - 1) / sms * (6 + 1) < (tiles + sms - 1) / sms * (8 * 6 + 3);
+}
+inline int fp64_tile(int nx, int ny, int sms)
+{
+    const long long big = (long long)((nx + 31) / 32) * ((ny + 7) / 8), small = (long long)((nx + 7) / 8) * ((ny + 3) / 4);
+    return fp64_small_tiles(big, small, sms) ? TILE_8x4 : TILE_32x8;
 }
 
 template <int N, class Pr>
@@ -30,7 +51,7 @@ cudaError_t launch_step(const KParams& P, const void* pin, void* pout, const voi
                         cudaStream_t st, TileRows rows = TileRows{ROWS_ALL, 0, 0});
 template <int N, class Pr>
 cudaError_t launch_export(const KParams& P, const void* pin, const void* ain, double* phi, double* T, double* H,
-                          double* fl, double* ux, double* uy, double* p, cudaStream_t st);
+                          double* fl, double* ux, double* uy, double* p, int tile, cudaStream_t st);
 template <int N, class Pr>
 cudaError_t launch_init(const KParams& P, const double* phi, const double* T, const double* ux, const double* uy,
                         void* pop, void* aux, cudaStream_t st);
@@ -64,6 +85,7 @@ cudaError_t launch_diag(const KParams& P, const void* pop, const void* aux, doub
 
 // ---- batches of independent cases (lbm_batch.cuh) -----------------------------------
 constexpr int BATCH_NT = 256;   // threads of every batch block (all batch tile shapes)
+constexpr int BATCH_SUB = 8;    // tiles of 8x4 in a batch tile of any shape
 
 struct BatchCase {
     const void* pop[2];
@@ -75,6 +97,8 @@ struct BatchCase {
 
 struct BatchTable {            // one group of cases sharing a tile shape
     int total_tiles;
+    long long total_subtiles;   // tiles of 8x4 that cover the same cases (FP64 per-step form)
+    int sms;
     const BatchCase* cases;     // [all cases of the batch]
     const KParams* params;      // [all cases of the batch]
     const int* tile_case;       // [total_tiles] case of each tile of the group, cases in order

@@ -151,7 +151,7 @@ bool message_rows(const lbm_handle* h, int side, int phase, bool pack, SlabRows&
 TileRows slab_rows(const lbm_handle* h, int part)
 {
     int tx = 32, ty = 8;
-    tile_dims(h->tile, tx, ty);
+    tile_dims(lbm_step_tile(h), tx, ty);
     const int tiles_y = (h->ny + ty - 1) / ty;
     const int lo = 1;                                              // rows >= ty, ring >= ty - 1 >= 2
     int hi = h->ny - 3 - ty >= 0 ? (h->ny - 3 - ty) / ty + 1 : 0;  // last row + 1 (ring) <= ny - 3
@@ -274,7 +274,7 @@ int lbm_slab_step_part(lbm_handle* h, int part)
                                                                    h->aux[a], h->aux[b], h->stage_status, h->stream,
                                                                    rows);
         return launch_step<decltype(n)::value, decltype(pr)>(h->P, h->pop[a], h->pop[b], h->aux[a], h->aux[b],
-                                                             h->tile, h->stream, rows);
+                                                             lbm_step_tile(h), h->stream, rows);
     });
     if (e != cudaSuccess) {
         cudaGetLastError();
