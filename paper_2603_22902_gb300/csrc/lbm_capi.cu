@@ -232,6 +232,7 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
     P.ny = grid->ny;
     P.N = N;
     P.S = (long long)grid->nx * grid->ny;
+    P.S32 = (unsigned)P.S;
     for (int s = 0; s < 4; ++s) {
         P.bc[s] = bc->kind[s];
         P.tbc[s] = bc->tkind[s];

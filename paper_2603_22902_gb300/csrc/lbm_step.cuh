@@ -94,28 +94,27 @@ __device__ __forceinline__ val_t<typename Pr::R> stored(T q)
 
 // Load population i of species s at cell c in its stored form.
 template <class Pr>
-__device__ __forceinline__ val_t<typename Pr::R> ld_val(const KParams& P, const PopView<Pr>& v, int s, int i, long long c, int site)
+__device__ __forceinline__ val_t<typename Pr::R> ld_val(const KParams& P, const PopView<Pr>& v, int s, int i, unsigned c, int site)
 {
-    if (i == 0) return stored<Pr>(LBM_LDX(Pr::COH, P, v.rest, (long long)s * P.S + c, P.rest_elems, site));
-    return stored<Pr>(LBM_LDX(Pr::COH, P, v.move, (long long)(s * 8 + i - 1) * P.S + c, P.move_elems, site));
+    if (i == 0) return stored<Pr>(ld_plane<Pr::COH>(P, v.rest, s, c, P.rest_elems, site));
+    return stored<Pr>(ld_plane<Pr::COH>(P, v.move, s * 8 + i - 1, c, P.move_elems, site));
 }
 
 // The same load for a second read of a population in one step: through the cached
 // (L1) path instead of the read-only one, so that the compiler does not merge it with
 // the first read and keep the value in a register meanwhile.
 template <class Pr>
-__device__ __forceinline__ val_t<typename Pr::R> ld_val_late(const KParams& P, const PopView<Pr>& v, int s, int i, long long c,
-                                                             int site)
+__device__ __forceinline__ val_t<typename Pr::R> ld_val_late(const KParams& P, const PopView<Pr>& v, int s, int i, unsigned c, int site)
 {
-    const long long idx = i == 0 ? (long long)s * P.S + c : (long long)(s * 8 + i - 1) * P.S + c;
 #ifdef LBM_CHECK_BOUNDS
+    const long long idx = i == 0 ? (long long)s * P.S + c : (long long)(s * 8 + i - 1) * P.S + c;
     if (!lbm_in_bounds(P.dbg, idx, i == 0 ? P.rest_elems : P.move_elems, site))
         return val_t<typename Pr::R>((typename Pr::R)0.0f);
 #else
     (void)site;
 #endif
-    if (i == 0) return stored<Pr>(lbm_ld_l1<Pr::COH>(v.rest + idx));
-    return stored<Pr>(lbm_ld_l1<Pr::COH>(v.move + idx));
+    if (i == 0) return stored<Pr>(lbm_ld_l1<Pr::COH>(plane_elem(v.rest, P, s, c)));
+    return stored<Pr>(lbm_ld_l1<Pr::COH>(plane_elem(v.move, P, s * 8 + i - 1, c)));
 }
 
 // Store the plain value val of population i of species s at cell c (quantised from R).
@@ -141,22 +140,19 @@ __device__ __forceinline__ void st_pop(const KParams& P, const PopView<Pr>& v, i
     }
 }
 
-// Store population i of species s at cell c from its stored form: the plain value, or for the
-// 16-bit policies f_i / (w_i F_SCALE), g_i / w_i, h_i / (w_i rho_ref c_p,ref) of a moving direction
-// and the plain value of the rest direction.
+// Store population i of species s at cell c + shift from its stored form: the plain value, or for
+// the 16-bit policies f_i / (w_i F_SCALE), g_i / w_i, h_i / (w_i rho_ref c_p,ref) of a moving direction
+// and the plain value of the rest direction.  shift is the same for all threads.
 template <class Pr>
-__device__ __forceinline__ void st_val(const KParams& P, const PopView<Pr>& v, int s, int i, long long c,
+__device__ __forceinline__ void st_val(const KParams& P, const PopView<Pr>& v, int s, int i, int shift, unsigned c,
                                        val_t<typename Pr::R> val, int site)
 {
     using R = typename Pr::R;
+    using TR = typename Pr::TR;
     using TM = typename Pr::TM;
-    if (i == 0) {
-        LBM_ST(P, v.rest, (long long)s * P.S + c, P.rest_elems, site, (typename Pr::TR)(R)val);
-        return;
-    }
-    const long long idx = (long long)(s * 8 + i - 1) * P.S + c;
-    if constexpr (!Pr::QUANT) LBM_ST(P, v.move, idx, P.move_elems, site, (TM)(R)val);
-    else LBM_ST(P, v.move, idx, P.move_elems, site, from_f<TM>((R)val));
+    if (i == 0) st_plane<TR>(P, v.rest, s, shift, c, P.rest_elems, site, (TR)(R)val);
+    else if constexpr (!Pr::QUANT) st_plane<TM>(P, v.move, s * 8 + i - 1, shift, c, P.move_elems, site, (TM)(R)val);
+    else st_plane<TM>(P, v.move, s * 8 + i - 1, shift, c, P.move_elems, site, from_f<TM>((R)val));
 }
 
 // Where a step reads its inputs.  A loader addresses a cell of the tile-with-ring by a
@@ -168,14 +164,12 @@ __device__ __forceinline__ void st_val(const KParams& P, const PopView<Pr>& v, i
 template <class Pr>
 struct GlobalLoader {
     using V = val_t<typename Pr::R>;
-    using Cell = long long;
+    using Cell = unsigned;
     static constexpr bool GLOBAL = true;   // step_tile_l locates the cells itself
     const KParams& P;
     PopView<Pr> pin;
     const typename Pr::TA* __restrict__ ain;
-    long long S;
-    int nx;
-    __device__ __forceinline__ Cell own(int x, int y, int, int) const { return (long long)y * nx + x; }
+    __device__ __forceinline__ Cell own(int x, int y, int, int) const { return (unsigned)y * (unsigned)P.nx + (unsigned)x; }
     __device__ __forceinline__ V pop(int s, int i, Cell c, int site) const { return ld_val<Pr>(P, pin, s, i, c, site); }
     __device__ __forceinline__ V pop_late(int s, int i, Cell c, int site) const
     {
@@ -183,7 +177,7 @@ struct GlobalLoader {
     }
     __device__ __forceinline__ V aux(int a, Cell c, int site) const
     {
-        return V((typename Pr::R)LBM_LDX(Pr::COH, P, ain, a * S + c, P.aux_elems, site));
+        return V((typename Pr::R)ld_plane<Pr::COH>(P, ain, a, c, P.aux_elems, site));
     }
 };
 
@@ -199,11 +193,11 @@ __device__ __forceinline__ void cell_moments(const KParams& P, const L& ld, type
 // phi_p, rho and psi of a cell (what its neighbours' stencils read).
 template <int N, class Pr>
 __device__ __forceinline__ void halo_moments(const KParams& P, const PopView<Pr>& pin,
-                                             const typename Pr::TA* __restrict__ ain, long long c,
+                                             const typename Pr::TA* __restrict__ ain, unsigned c,
                                              val_t<typename Pr::R> (&phi)[N], val_t<typename Pr::R>& rho,
                                              val_t<typename Pr::R>& psi)
 {
-    const GlobalLoader<Pr> ld{P, pin, ain, P.S, P.nx};
+    const GlobalLoader<Pr> ld{P, pin, ain};
     val_t<typename Pr::R> rhoH, fl;
     cell_moments<N, Pr>(P, ld, c, phi, rhoH, fl);
     mix_rho_psi<N>(P, phi, fl, rho, psi);
@@ -227,15 +221,15 @@ __device__ __forceinline__ void push(const KParams& P, const PopView<Pr>& out, i
         if (P.bc[2] == PERIODIC) ty = ty < 0 ? ty + P.ny : ty - P.ny;
         else yo = true;
     }
-    const long long own = (long long)y * P.nx + x;
+    const unsigned own = (unsigned)y * (unsigned)P.nx + (unsigned)x;
     if (!xo && !yo) {
-        st_val<Pr>(P, out, s, J, (long long)ty * P.nx + tx, q, 10);
+        st_val<Pr>(P, out, s, J, 0, (unsigned)ty * (unsigned)P.nx + (unsigned)tx, q, 10);
     } else if (xo) {
-        st_val<Pr>(P, out, s, opp(J), own, q, 11);
+        st_val<Pr>(P, out, s, opp(J), 0, own, q, 11);
     } else {
         const int side = ty < 0 ? 2 : 3;
         if (P.bc[side] == WALL && !(KIND == KIND_H && P.tbc[side] == DIRICHLET))
-            st_val<Pr>(P, out, s, opp(J), own, q, 12);
+            st_val<Pr>(P, out, s, opp(J), 0, own, q, 12);
     }
 }
 
@@ -250,7 +244,7 @@ __device__ __forceinline__ void push_row(const KParams& P, const PopView<Pr>& ou
         if (P.bc[0] != PERIODIC) return;
         tx = tx < 0 ? tx + P.nx : tx - P.nx;
     }
-    st_val<Pr>(P, out, s, J, (long long)y * P.nx + tx, v, 13);
+    st_val<Pr>(P, out, s, J, 0, (unsigned)y * (unsigned)P.nx + (unsigned)tx, v, 13);
 }
 
 // push_row for a direction j known at run time, whose x component is dx.
@@ -263,36 +257,26 @@ __device__ __forceinline__ void push_row_at(const KParams& P, const PopView<Pr>&
         if (P.bc[0] != PERIODIC) return;
         tx = tx < 0 ? tx + P.nx : tx - P.nx;
     }
-    st_val<Pr>(P, out, s, j, (long long)y * P.nx + tx, v, 13);
+    st_val<Pr>(P, out, s, j, 0, (unsigned)y * (unsigned)P.nx + (unsigned)tx, v, 13);
 }
 
-// All nine pushes of one species, plus the outflow copies of the boundary rows.  Three
-// paths, chosen per cell by the caller:
-//   PUSH_INTERIOR: the cell's row is neither the lattice's first nor its last, and its
-//     tile's columns and their ring lie inside the lattice: every population lands in the
-//     neighbour c + c_J, no wrap and no boundary rule;
-//   PUSH_XWRAP: the cell's row is neither the first nor the last, and x is periodic: the
-//     neighbour c + c_J with its x taken modulo nx, no boundary rule;
-//   PUSH_GENERAL: the checks of push() for every population.
-constexpr int PUSH_GENERAL = 0, PUSH_INTERIOR = 1, PUSH_XWRAP = 2;
+// All nine pushes of one species, plus the outflow copies of the boundary rows.  Two paths,
+// chosen per cell by the caller:
+//   inside: the cell's row is neither the lattice's first nor its last, and x is periodic or the
+//     columns of its tile and their ring lie inside the lattice: every population lands in
+//     the neighbour c + c_J with its x taken modulo nx, no boundary rule;
+//   otherwise the checks of push() for every population.
 template <int KIND, class Pr>
 __device__ __forceinline__ void push_species(const KParams& P, const PopView<Pr>& out, int s, int x, int y,
-                                             int path, const val_t<typename Pr::R> (&q)[9])
+                                             bool inside, const val_t<typename Pr::R> (&q)[9])
 {
-    if (path == PUSH_INTERIOR) {
-        const long long c = (long long)y * P.nx + x;
-        st_val<Pr>(P, out, s, 0, c, q[0], 10);
-#pragma unroll
-        for (int j = 1; j < 9; ++j) st_val<Pr>(P, out, s, j, c + (cy(j) * P.nx + cx(j)), q[j], 10);
-        return;
-    }
-    if (path == PUSH_XWRAP) {
-        const long long row = (long long)y * P.nx;
-        const int xm = x == 0 ? P.nx - 1 : x - 1, xp = x == P.nx - 1 ? 0 : x + 1;
-        st_val<Pr>(P, out, s, 0, row + x, q[0], 10);
+    if (inside) {
+        const unsigned nx = (unsigned)P.nx, c = (unsigned)y * nx + (unsigned)x;
+        const unsigned cm = x == 0 ? c + (nx - 1) : c - 1, cp = x == P.nx - 1 ? c - (nx - 1) : c + 1;
+        st_val<Pr>(P, out, s, 0, 0, c, q[0], 10);
 #pragma unroll
         for (int j = 1; j < 9; ++j)
-            st_val<Pr>(P, out, s, j, row + cy(j) * P.nx + (cx(j) < 0 ? xm : (cx(j) > 0 ? xp : x)), q[j], 10);
+            st_val<Pr>(P, out, s, j, cy(j) * P.nx, cx(j) < 0 ? cm : (cx(j) > 0 ? cp : c), q[j], 10);
         return;
     }
     push<0, KIND, Pr>(P, out, s, x, y, q[0]);
@@ -344,8 +328,9 @@ struct CellIo {
     const PopView<Pr>& pout;
     TA* __restrict__ aout;
     const ExportPtrs& ex;
-    int lx, ly, x, y, path;
-    long long c;
+    int lx, ly, x, y;
+    bool inside;                   // push_species
+    unsigned c;
     typename L::Cell oc;
     __device__ __forceinline__ void stencil(int fi, V& gx, V& gy, V& lap) const
     {
@@ -362,11 +347,11 @@ struct CellIo {
     template <int KIND>
     __device__ __forceinline__ void push(int s, const V (&q)[9])
     {
-        push_species<KIND, Pr>(P, pout, s, x, y, path, q);
+        push_species<KIND, Pr>(P, pout, s, x, y, inside, q);
     }
     __device__ __forceinline__ void put_lag(int a, V v)
     {
-        LBM_ST(P, aout, a * P.S + c, P.aux_elems, 30, (TA)(typename Pr::R)v);
+        st_plane<TA>(P, aout, a, 0, c, P.aux_elems, 30, (TA)(typename Pr::R)v);
     }
     // Dirichlet wall: ghost behind the half-way wall with T_g = 2 T_w - T, u = 0; its
     // post-collision population is h_eq(ghost) + (1 - 1/tau_h)(h_j - h_eq_j) for the
@@ -502,7 +487,7 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
                 if (yper) gy = wrap_index(gy, ny);
                 else { beyond = true; gy = min(max(gy, 0), ny - 1); }
             }
-            cell = (long long)gy * nx + gx;
+            cell = (unsigned)gy * (unsigned)nx + (unsigned)gx;
             return !beyond;
         } else {
             return ld.locate(lx, ly, cell);
@@ -575,12 +560,9 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
     // the push path of this cell (push_species): the same for a row of the tile, so for a
     // warp of a 32-wide tile; only the lattice's first and last rows, and columns at a
     // side that is not periodic, take the general path
-    const bool row_inside = y >= 1 && y <= ny - 2;
-    const int path = row_inside && x0 >= 1 && x0 + TX <= nx - 1 ? PUSH_INTERIOR
-                     : row_inside && xper                         ? PUSH_XWRAP
-                                                                  : PUSH_GENERAL;
+    const bool inside = y >= 1 && y <= ny - 2 && (xper || (x0 >= 1 && x0 + TX <= nx - 1));
     const PopView<Pr> pout = pop_view<Pr>(P, pout_base);
-    CellIo<N, H, W, Pr, L> io{P, ld, fields, pout, aout, ex, tx + 1, ty + 1, x, y, path, (long long)y * nx + x,
+    CellIo<N, H, W, Pr, L> io{P, ld, fields, pout, aout, ex, tx + 1, ty + 1, x, y, inside, (unsigned)y * (unsigned)nx + (unsigned)x,
                               ld.own(x, y, tx, ty)};
     cell_update<N, COLLIDE, Pr>(P, io, phi, rhoH, fl);
 }
@@ -592,7 +574,7 @@ __device__ __forceinline__ void step_tile(const KParams& P, const void* __restri
                                           typename Pr::TA* __restrict__ aout, const ExportPtrs& ex, int bx, int by,
                                           typename Pr::R* smem)
 {
-    const GlobalLoader<Pr> ld{P, pop_view<Pr>(P, pin_base), ain, P.S, P.nx};
+    const GlobalLoader<Pr> ld{P, pop_view<Pr>(P, pin_base), ain};
     step_tile_l<N, TX, TY, COLLIDE, Pr>(P, ld, pout_base, aout, ex, bx, by, smem);
 }
 
