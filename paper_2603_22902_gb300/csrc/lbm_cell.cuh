@@ -469,14 +469,15 @@ __device__ __forceinline__ void cell_update(const KParams& P, Io& io, const V (&
         const V rom = oms * rho, krho = ks * rho;
         const V hrom = rom * K(0.5), kFx = ks * Fx, kFy = ks * Fy;
         const V X = rfma(hrom, ux, kFx), Y = rfma(hrom, uy, kFy);
-        const V ayy = ey * Y, axy = rfma(ex, Y, ey * X);
-        const V s = (ks * S) * cst<V>(SC ? 1.5 : 1.0 / 6.0);
+        const V axy = rfma(ex, Y, ey * X);
+        const V kS = ks * S;
+        const auto cs = cst<V>(SC ? 1.5 : 1.0 / 6.0);
         const V omp = oms * p;
-        const V iso = rfma(ex, X, ayy) * cst<V>(-1.0 / 3.0);
+        const V iso = rfma(ex, X, ey * Y) * cst<V>(-1.0 / 3.0);
         const V a0 = rfma(omp, cst<V>(SC ? 3.0 : 1.0 / 3.0), iso);
         const V x0 = rfma(omp, cst<V>(SC ? -3.75 : -3.75 / 9.0), iso);
         const V tx = rfma(krho, fpx, rfma(rom, ux, kFx)), ty = rfma(krho, fpy, rfma(rom, uy, kFy));
-        const V as = a0 + s, bx = rfma(ex, X, as), by = as + ayy, bd = (bx + ayy) + s;
+        const V as = rfma(kS, cs, a0), bx = rfma(ex, X, as), by = rfma(ey, Y, as), bd = rfma(kS, cs, rfma(ey, Y, bx));
         V q[9];
         q[0] = rfma(x0, rest_weight<SC, V>(F_SCALE), om1 * f[0]);
         collide_pairs<SC>(om1, f, bx, by, bd + axy, bd - axy, tx, ty, cst<V>(SC ? 3.0 : 1.0 / 3.0), q);

@@ -303,8 +303,9 @@ __device__ __forceinline__ void staged_tile_issue(const StageMaps& M, int bx, in
         const unsigned bar = smem_addr(dyn + Lay::OBAR);
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        stage_issue<N, Pr>(M, dyn, bar, bx, by);
     }
+    step_wait_previous();
+    if (threadIdx.x == 0) stage_issue<N, Pr>(M, dyn, smem_addr(dyn + Lay::OBAR), bx, by);
 }
 
 template <int N, class Pr>

@@ -548,6 +548,7 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
     }
     __syncthreads();
     fill_ghosts<N, TX, TY, NT>(P, fields, x0, y0);
+    if constexpr (!Pr::COH) step_launch_next();
     if (!owned) return;
     if constexpr (Pr::COMPACT) {
 #pragma unroll
@@ -631,6 +632,7 @@ fused_step_kernel(const KParams P, const void* __restrict__ pin_base, void* __re
     __shared__ typename Pr::R smem[tile_smem_elems<N, TX, TY, Pr>()];
     int bx, by;
     tile_of_block(blockIdx.x, (P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY, rows, bx, by);
+    step_wait_previous();
     step_tile<N, TX, TY, COLLIDE, Pr>(P, pin_base, pout_base, ain, aout, ex, bx, by, smem);
 }
 
