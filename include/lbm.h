@@ -354,7 +354,7 @@ typedef struct {
  *   reverse sweep recomputes one segment at a time from its checkpoint, stores its
  *   states, and steps the adjoint back through them.
  * - Device memory: (nsteps / checkpoint_every + checkpoint_every + 2) states plus
- *   20 + 11 N planes of doubles, allocated for the duration of the call.
+ *   21 + 11 N planes of doubles, allocated for the duration of the call.
  * - FP64 handles only (LBM_EINVAL otherwise). fl_target and weight are [ny][nx] like
  *   the fields, in host or device memory per `where`.
  * - On return the handle holds the state after nsteps steps. Synchronises. */

@@ -4,7 +4,7 @@
 // One step maps set A (populations f, g_p, h and the lagged planes) to set B.  Its
 // adjoint maps the adjoint of set B (A-bar_{n+1}) to that of set A (A-bar_n), and adds
 // the step's share of the parameter gradients.  It runs in three kernels:
-//   1. mac_kernel: phi_p, rho, psi of every cell of A (the stencil inputs), FP64 planes;
+//   1. mac_kernel: phi_p, rho, psi (the stencil inputs) and rho H of every cell of A, FP64 planes;
 //   2. adj_cell_kernel: per cell x, the step of x recomputed, then reversed from the
 //      adjoints of everything x wrote (its pushed populations, gathered from A-bar_{n+1}
 //      through the same boundary rules, and its lagged outputs).  It writes the adjoint
@@ -19,6 +19,12 @@
 // forward step took, as do the guards of the pairwise normals (a zero normal has zero
 // derivative).  Apart from ill-conditioned normals in the far tails of nearly absent
 // phases (ADJ_NORMAL_COND below), the result is the exact derivative of the discrete step.
+//
+// All three are bound by the FP64 unit.  A cell that eq. H calls liquid or solid uses that state's
+// coefficients alone, its moments come from mac_kernel's planes (so the cell kernel reads no
+// phase-field population), its quotients from one reciprocal, and the stencil adjoints of a cell away
+// from the sides go straight to their planes.  256 x 256, N = 4, us per launch, before and after:
+// mac 18 / 12, cell 306 / 272, moments 59 / 40.
 //
 // Parameter gradients accumulate per cell in FP64 planes (slot layout below) and are
 // reduced once at the end, in a fixed order.
@@ -44,10 +50,14 @@ __device__ __forceinline__ int dir_of(int dx, int dy)
     return 0;
 }
 
-// Target slot of the push of q_J from (x, y) (the rules of push()): false when dropped.
+// Target slot of the push of q_J from (x, y) (the rules of push()): false when dropped (cell and slot
+// are then the node's own, so that a load from them, issued ahead of the test, stays inside).
 template <int KIND>
 __device__ __forceinline__ bool push_target(const KParams& P, int J, int x, int y, long long& cell, int& slot)
 {
+    const long long own = (long long)y * P.nx + x;
+    cell = own;
+    slot = opp(J);
     int tx = x + cx(J), ty = y + cy(J);
     bool xo = false, yo = false;
     if (cx(J) != 0 && (unsigned)tx >= (unsigned)P.nx) {
@@ -58,30 +68,21 @@ __device__ __forceinline__ bool push_target(const KParams& P, int J, int x, int 
         if (P.bc[2] == PERIODIC) ty = ty < 0 ? ty + P.ny : ty - P.ny;
         else yo = true;
     }
-    const long long own = (long long)y * P.nx + x;
     if (!xo && !yo) {
         cell = (long long)ty * P.nx + tx;
         slot = J;
         return true;
     }
-    if (xo) {
-        cell = own;
-        slot = opp(J);
-        return true;
-    }
+    if (xo) return true;
     const int side = ty < 0 ? 2 : 3;
-    if (P.bc[side] == WALL && !(KIND == KIND_H && P.tbc[side] == DIRICHLET)) {
-        cell = own;
-        slot = opp(J);
-        return true;
-    }
-    return false;
+    return P.bc[side] == WALL && !(KIND == KIND_H && P.tbc[side] == DIRICHLET);
 }
 
 // Target of a boundary-row write (push_row): slot J of (x + c_J, y); false beyond an x wall.
 __device__ __forceinline__ bool row_target(const KParams& P, int J, int x, int y, long long& cell)
 {
     int tx = x + cx(J);
+    cell = (long long)y * P.nx + x;
     if (cx(J) != 0 && (unsigned)tx >= (unsigned)P.nx) {
         if (P.bc[0] != PERIODIC) return false;
         tx = tx < 0 ? tx + P.nx : tx - P.nx;
@@ -90,31 +91,82 @@ __device__ __forceinline__ bool row_target(const KParams& P, int J, int x, int y
     return true;
 }
 
+// Loads that a condition guards (a neighbour that may lie beyond a side, a weight that may be absent)
+// are lbm_ld_ca, which the compiler does not issue ahead of the condition, and their addresses
+// lie inside the planes either way.
+// The cells c + c_k of an inner cell (x, y), one whose neighbours lie neither beyond nor across a
+// side; the cell itself, nine times, for any other: a load of an inner cell's neighbour may be
+// issued ahead of the branch that guards it, so no address outside the planes is formed.
+struct Neighbours {
+    bool inner;
+    unsigned c[9];
+    __device__ __forceinline__ Neighbours(const KParams& P, int x, int y)
+    {
+        inner = x >= 1 && x <= P.nx - 2 && y >= 1 && y <= P.ny - 2;
+        const unsigned own = (unsigned)y * (unsigned)P.nx + (unsigned)x;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) c[k] = inner ? own + (unsigned)(cy(k) * P.nx + cx(k)) : own;
+    }
+};
+
 // Adjoint of everything cell (x, y) wrote for species s (KIND) from its nine pushes
 // (plus the outflow row copies of the same values).
 template <int KIND>
 __device__ __forceinline__ void gather_species(const KParams& P, const double* bpop, int s, int x, int y,
-                                               double (&qb)[9])
+                                               const Neighbours& nb, double (&qb)[9])
 {
+    if (nb.inner) {
+        qb[0] = lbm_ld_ca(plane_elem(bpop, P, s, nb.c[0]));
+#pragma unroll
+        for (int j = 1; j < 9; ++j) qb[j] = lbm_ld_ca(plane_elem(bpop + P.rest_elems, P, s * 8 + j - 1, nb.c[j]));
+        return;
+    }
     for (int j = 0; j < 9; ++j) {
         long long cell;
         int slot;
-        qb[j] = push_target<KIND>(P, j, x, y, cell, slot) ? bpop[pidx(P, s, slot, cell)] : 0.0;
+        qb[j] = push_target<KIND>(P, j, x, y, cell, slot) ? lbm_ld_ca(bpop + pidx(P, s, slot, cell)) : 0.0;
     }
     if (y == 0 && P.bc[2] == OUTFLOW) {
         const int js[3] = {2, 5, 6};
         for (int m = 0; m < 3; ++m) {
             long long cell;
-            if (row_target(P, js[m], x, y, cell)) qb[js[m]] += bpop[pidx(P, s, js[m], cell)];
+            if (row_target(P, js[m], x, y, cell)) qb[js[m]] += lbm_ld_ca(bpop + pidx(P, s, js[m], cell));
         }
     }
     if (y == P.ny - 1 && P.bc[3] == OUTFLOW) {
         const int js[3] = {4, 7, 8};
         for (int m = 0; m < 3; ++m) {
             long long cell;
-            if (row_target(P, js[m], x, y, cell)) qb[js[m]] += bpop[pidx(P, s, js[m], cell)];
+            if (row_target(P, js[m], x, y, cell)) qb[js[m]] += lbm_ld_ca(bpop + pidx(P, s, js[m], cell));
         }
     }
+}
+
+// The branch of eq. H that the forward map takes, as liquid_fraction decides it (an FP32 screen,
+// then the FP64 map), and f_l.
+constexpr int EQH_SOLID = 0, EQH_LIQUID = 1, EQH_MUSHY = 2, EQH_POINT = 3;   // POINT: f_l = 1, T = T_liq
+template <int N>
+__device__ __forceinline__ int eqh_branch(const KParams& P, const double (&phi)[N], double rhoH, double& fl)
+{
+    d1 ph[N];
+#pragma unroll
+    for (int p = 0; p < N; ++p) ph[p] = phi[p];
+    const int sure = eqh_screen<N>(P, ph, d1(rhoH));
+    if (sure >= 0) {
+        fl = sure;
+        return sure;
+    }
+    const Mix<N> m = mixture_map<N>(P, phi);
+    const double As = m.rs * m.cs * P.T_sol, Al = fma(m.rl * m.cl, P.T_liq, m.Lv);
+    fl = 1.0;
+    if (!(m.Lv > 0.0) || (!(rhoH < As) && rhoH > Al)) return EQH_LIQUID;
+    if (rhoH < As) {
+        fl = 0.0;
+        return EQH_SOLID;
+    }
+    if (!(Al - As > 0.0)) return EQH_POINT;
+    fl = (rhoH - As) / (Al - As);
+    return EQH_MUSHY;
 }
 
 // Reverse of eq. H: adjoints (fl_b, T_b) of the outputs -> adjoints of the mixture sums
@@ -165,23 +217,28 @@ __device__ __forceinline__ void map_reverse(const KParams& P, const Mix<N>& m, d
 // loss itself does not change, so the derivative through n is not followed.
 constexpr double ADJ_NORMAL_COND = 10.0;
 
+// Threads of a block of the adjoint kernels: the FP64 unit of the fullest SM sets the time, so
+// small blocks (256 x 256: 1024 of 64 threads, 6.7 to an SM, against 512 of 128, 3.4).
+constexpr int ADJ_NT = 64;
+
 // g'(x) and g''(x) of g(x) = x^2 (1 - x)^2.
 __device__ __forceinline__ double gp1(double x) { return 2.0 * x * (1.0 - x) * (1.0 - 2.0 * x); }
 __device__ __forceinline__ double gp2(double x) { return 2.0 - 12.0 * x + 12.0 * x * x; }
 
-// phi_p, rho, psi of every cell of set A (the inputs of the stencils).
+// phi_p, rho, psi of every cell of set A (the inputs of the stencils), and rho H.
 template <int N>
-__global__ void mac_kernel(const KParams P, const double* __restrict__ pin, const double* __restrict__ ain,
+__global__ void __launch_bounds__(ADJ_NT) mac_kernel(const KParams P, const double* __restrict__ pin, const double* __restrict__ ain,
                            double* __restrict__ mac)
 {
     const PopView<PrecFP64> pv = pop_view<PrecFP64>(P, pin);
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < P.S;
          c += (long long)gridDim.x * blockDim.x) {
-        d1 ph[N], r, ps;
-        halo_moments<N, PrecFP64>(P, pv, ain, c, ph, r, ps);
+        d1 ph[N], r, ps, rH;
+        halo_moments<N, PrecFP64>(P, pv, ain, c, ph, r, ps, rH);
         for (int p = 0; p < N; ++p) mac[p * P.S + c] = ph[p].v;
         mac[N * P.S + c] = r.v;
         mac[(N + 1) * P.S + c] = ps.v;
+        mac[(N + 2) * P.S + c] = rH.v;
     }
 }
 
@@ -218,7 +275,7 @@ __device__ __forceinline__ void stencil_source(const KParams& P, int x, int y, i
 
 // The adjoint of one cell's step (see the file comment).
 template <int N>
-__global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const AdjBufs B)
+__global__ void __launch_bounds__(ADJ_NT) adj_cell_kernel(const KParams P, const AdjBufs B)
 {
     const long long S = P.S;
     const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -226,77 +283,82 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
     const int x = (int)(c % P.nx), y = (int)(c / P.nx);
     const Coef<double>& C = P.d;
 
+    const Neighbours nb(P, x, y);
+
     // ================= forward recompute (the FP64 step of cell c) =================
-    double f[9], g[N][9], h[9];
+    double f[9], h[9];
     for (int i = 0; i < 9; ++i) {
         f[i] = B.pin[pidx(P, 0, i, c)];
         h[i] = B.pin[pidx(P, N + 1, i, c)];
-        for (int p = 0; p < N; ++p) g[p][i] = B.pin[pidx(P, 1 + p, i, c)];
     }
-    const double mdm = B.ain[aux_mdot() * S + c], Qm = B.ain[aux_Q() * S + c];
     const double psim = B.ain[aux_psi() * S + c];
-    const double iden = 1.0 / (1.0 - 0.5 * mdm);
     double phi[N];
-    for (int p = 0; p < N; ++p) {
-        double sg = 0.0;
-        for (int i = 0; i < 9; ++i) sg += g[p][i];
-        phi[p] = sg * iden;
-    }
-    double sh = 0.0;
-    for (int i = 0; i < 9; ++i) sh += h[i];
-    const double rhoH = fma(0.5, Qm, sh);
-    const Mix<N> m = mixture_map<N>(P, phi);
-    double fl, T;
-    enthalpy_map<N, true>(P, m, rhoH, fl, T);
+    for (int p = 0; p < N; ++p) phi[p] = B.mac[p * S + c];
+    const double rho = B.mac[N * S + c], psi = B.mac[(N + 1) * S + c], rhoH = B.mac[(N + 2) * S + c];
+    // eq. H and eq. 2: a cell that is wholly liquid or solid needs that state's coefficients alone
+    double fl;
+    const int branch = eqh_branch<N>(P, phi, rhoH, fl);
+    const bool pure = branch == EQH_LIQUID || branch == EQH_SOLID, solid = branch == EQH_SOLID;
     const double fs = 1.0 - fl;
-    const double Rs = mix_sum<N, double>(phi, C.rho_s), Rl = mix_sum<N, double>(phi, C.rho_l);
-    const double Ms = mix_sum<N, double>(phi, C.mu_s), Ml = mix_sum<N, double>(phi, C.mu_l);
-    const double Ks = mix_sum<N, double>(phi, C.lam_s), Kl = mix_sum<N, double>(phi, C.lam_l);
-    const double Cs = mix_sum<N, double>(phi, C.cp_s), Cl = mix_sum<N, double>(phi, C.cp_l);
-    const double Dr = mix_sum<N, double>(phi, C.drho), Pc = mix_sum<N, double>(phi, C.pcm);
-    const double rho = fma(fs, Rs, fl * Rl), mu = fma(fs, Ms, fl * Ml);
-    const double lam = fma(fs, Ks, fl * Kl), cp = fma(fs, Cs, fl * Cl);
-    const double psi = fs * Dr, chi = fs * Pc;
+    double mu, lam, cp, chi;
+    if (pure) {
+        mu = mix_sum<N, double>(phi, solid ? C.mu_s : C.mu_l);
+        lam = mix_sum<N, double>(phi, solid ? C.lam_s : C.lam_l);
+        cp = mix_sum<N, double>(phi, solid ? C.cp_s : C.cp_l);
+        chi = solid ? mix_sum<N, double>(phi, C.pcm) : 0.0;
+    } else {
+        mu = fma(fs, mix_sum<N, double>(phi, C.mu_s), fl * mix_sum<N, double>(phi, C.mu_l));
+        lam = fma(fs, mix_sum<N, double>(phi, C.lam_s), fl * mix_sum<N, double>(phi, C.lam_l));
+        cp = fma(fs, mix_sum<N, double>(phi, C.cp_s), fl * mix_sum<N, double>(phi, C.cp_l));
+        chi = fs * mix_sum<N, double>(phi, C.pcm);
+    }
 
     // stencil values (ghosts beyond walls / outflows as in the forward step)
-    double vphi[9][N], vrho[9], vpsi[9];
-    int ksrc[9], wxk[9], wyk[9];
-    for (int k = 0; k < 9; ++k) {
-        long long sc;
-        stencil_source(P, x, y, k, sc, ksrc[k], wxk[k], wyk[k]);
-        double ph[N];
-        for (int p = 0; p < N; ++p) ph[p] = B.mac[p * S + sc];
-        for (int p = 0; p < N; ++p) {
-            double corr = 0.0;
-            if (wxk[k] >= 0 || wyk[k] >= 0)
-                for (int q = 0; q < N; ++q) {
-                    if (q == p) continue;
-                    double cw = 0.0;
-                    if (wxk[k] >= 0) cw += C.wet[wxk[k]][p][q];
-                    if (wyk[k] >= 0) cw += C.wet[wyk[k]][p][q];
-                    corr = fma(cw * ph[p], ph[q], corr);
-                }
-            vphi[k][p] = ph[p] + corr;
-        }
-        vrho[k] = B.mac[N * S + sc];
-        vpsi[k] = B.mac[(N + 1) * S + sc];
-    }
-    // the own cell's stencil centre is its own value (it is the same computation)
     auto gradv = [&](const double* v, double& gx_, double& gy_) {
-        gx_ = (v[1] - v[3]) * (1.0 / 3.0) + ((v[5] - v[6]) + (v[8] - v[7])) * (1.0 / 12.0);
-        gy_ = (v[2] - v[4]) * (1.0 / 3.0) + ((v[5] - v[8]) + (v[6] - v[7])) * (1.0 / 12.0);
+        const double d1_ = v[5] - v[7], d2_ = v[6] - v[8];
+        gx_ = fma(4.0, v[1] - v[3], d1_ - d2_) * (1.0 / 12.0);
+        gy_ = fma(4.0, v[2] - v[4], d1_ + d2_) * (1.0 / 12.0);
     };
-    double gpx[N], gpy[N], lap[N];
-    for (int p = 0; p < N; ++p) {
+    double gpx[N], gpy[N], lap[N], grx, gry, gsx, gsy;
+#pragma unroll
+    for (int fld = 0; fld < N + 2; ++fld) {
         double v[9];
-        for (int k = 0; k < 9; ++k) v[k] = vphi[k][p];
-        gradv(v, gpx[p], gpy[p]);
-        lap[p] = ((v[1] + v[3]) + (v[2] + v[4])) * (2.0 / 3.0) + ((v[5] + v[6]) + (v[8] + v[7])) * (1.0 / 6.0) -
-                 v[0] * (10.0 / 3.0);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            if (nb.inner) {
+                v[k] = lbm_ld_ca(plane_elem(B.mac, P, fld, nb.c[k]));
+            } else {
+                long long sc;
+                int ks, wx, wy;
+                stencil_source(P, x, y, k, sc, ks, wx, wy);
+                v[k] = lbm_ld_ca(B.mac + fld * S + sc);
+                if (fld < N && (wx >= 0 || wy >= 0)) {
+                    double corr = 0.0;
+                    for (int q = 0; q < N; ++q) {
+                        if (q == fld) continue;
+                        double cw = 0.0;
+                        if (wx >= 0) cw += C.wet[wx][fld][q];
+                        if (wy >= 0) cw += C.wet[wy][fld][q];
+                        corr = fma(cw * v[k], lbm_ld_ca(B.mac + q * S + sc), corr);
+                    }
+                    v[k] += corr;
+                }
+            }
+        }
+        double gx_, gy_;
+        gradv(v, gx_, gy_);
+        if (fld < N) {
+            gpx[fld] = gx_;
+            gpy[fld] = gy_;
+            lap[fld] = fma(((v[1] + v[3]) + (v[2] + v[4])), 2.0 / 3.0, fma((v[5] + v[7]) + (v[6] + v[8]), 1.0 / 6.0, v[0] * (-10.0 / 3.0)));
+        } else if (fld == N) {
+            grx = gx_;
+            gry = gy_;
+        } else {
+            gsx = gx_;
+            gsy = gy_;
+        }
     }
-    double grx, gry, gsx, gsy;
-    gradv(vrho, grx, gry);
-    gradv(vpsi, gsx, gsy);
 
     // stage D
     constexpr int NP = N * (N - 1) / 2;
@@ -353,7 +415,12 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
     const double sum_f = ((f[1] + f[2]) + (f[3] + f[4])) + ((f[5] + f[6]) + (f[7] + f[8]));
     const double Af = fma(3.0, mu, 0.5 * rho);
     const double Bh = fma(lam, C.tau_h_scale, 0.5);
-    const double irho = 1.0 / rho, om = rho / Af, oh = 1.0 / Bh;
+    // 1 / rho, omega_f, omega_h and 1 / (rho c_p) from one reciprocal
+    const double RA = rho * Af, BC = Bh * cp;
+    const double rr = 1.0 / (RA * BC), rRA = BC * rr, rBC = RA * rr;
+    const double irho = Af * rRA, om = rho * rho * rRA, oh = cp * rBC, icr = irho * (Bh * rBC);
+    const double Zsens = solid ? rhoH : rhoH - mix_sum<N, double>(phi, C.rhoL);   // pure cells: rho c_p T
+    const double T = pure ? Zsens * icr : branch == EQH_MUSHY ? fma(fl, P.T_liq - P.T_sol, P.T_sol) : P.T_liq;
     const double usx = fma(0.5, Fx, jx) * irho, usy = fma(0.5, Fy, jy) * irho;
     const double fpx = chi * (C.us[0] - usx), fpy = chi * (C.us[1] - usy);
     const double ux = fma(0.5, fpx, usx), uy = fma(0.5, fpy, usy);
@@ -379,11 +446,8 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
     const double ohZ = oh * Z;
 
     // ======================= reverse =======================
-    double f_b[9], g_b[N][9], h_b[9];
-    for (int i = 0; i < 9; ++i) {
-        f_b[i] = h_b[i] = 0.0;
-        for (int p = 0; p < N; ++p) g_b[p][i] = 0.0;
-    }
+    double f_b[9], h_b[9];
+    for (int i = 0; i < 9; ++i) f_b[i] = h_b[i] = 0.0;
     double phi_b[N], Rx_b[N], Ry_b[N], mup_b[N], gpx_b[N], gpy_b[N], lap_b[N], gpv_b[N];
     for (int p = 0; p < N; ++p) phi_b[p] = Rx_b[p] = Ry_b[p] = mup_b[p] = gpx_b[p] = gpy_b[p] = lap_b[p] = gpv_b[p] = 0.0;
     double rho_b = 0, mu_b = 0, lam_b = 0, cp_b = 0, psi_b = 0, chi_b = 0, T_b = 0, rhoH_b = 0;
@@ -399,7 +463,7 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
     // ---- enthalpy collision ----
     {
         double qb[9];
-        gather_species<KIND_H>(P, B.bpop, N + 1, x, y, qb);
+        gather_species<KIND_H>(P, B.bpop, N + 1, x, y, nb, qb);
         double Z_b = 0, E_b = 0, kh_b = 0, oh1_b = 0, ohZ_b = 0;
         // Dirichlet rows: v_j = oh1 (h_j - heq_j) + w_j Eg, Eg = E_ref (2 T_w - T)
         auto dirichlet = [&](int side, int j0, int j1, int j2) {
@@ -409,7 +473,7 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
                 const int j = js[mm];
                 long long cell;
                 if (!row_target(P, j, x, y, cell)) continue;
-                const double vb = B.bpop[pidx(P, N + 1, j, cell)];
+                const double vb = lbm_ld_ca(B.bpop + pidx(P, N + 1, j, cell));
                 const double cu = cx(j) * ux + cy(j) * uy;
                 const double Pj = fma(4.5 * cu, cu, fma(3.0, cu, -1.5 * uu));
                 const double heq = wgt(j) * fma(Z, Pj, E);
@@ -483,8 +547,9 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
     // ---- phase-field collisions ----
     for (int pp = 0; pp < N; ++pp) {
         double qb[9];
-        gather_species<KIND_G>(P, B.bpop, 1 + pp, x, y, qb);
-        for (int i = 0; i < 9; ++i) g_b[pp][i] += og1 * qb[i];
+        gather_species<KIND_G>(P, B.bpop, 1 + pp, x, y, nb, qb);
+        // (the adjoint of the moments is added by adj_moments_kernel)
+        for (int i = 0; i < 9; ++i) B.apop[pidx(P, 1 + pp, i, c)] = og1 * qb[i];
         double wq[9];
         for (int i = 0; i < 9; ++i) wq[i] = wgt(i) * qb[i];
         const double b0_b = wq[0] + wq[1] + wq[2] + wq[3] + wq[4] + wq[5] + wq[6] + wq[7] + wq[8];
@@ -514,7 +579,7 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
     // ---- flow collision ----
     {
         double qb[9];
-        gather_species<KIND_F>(P, B.bpop, 0, x, y, qb);
+        gather_species<KIND_F>(P, B.bpop, 0, x, y, nb, qb);
         double Xb[9], om1_b = 0.0;
         for (int i = 0; i < 9; ++i) {
             f_b[i] += om1 * qb[i];
@@ -632,7 +697,7 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
         f_b[4] -= jy_b;
         // irho = 1/rho, om = rho / Af, oh = 1 / Bh; Af = 3 mu + rho/2, Bh = lam tau_s + 1/2
         rho_b += -irho * irho * irho_b;
-        const double iAf = 1.0 / Af;
+        const double iAf = om * irho;
         rho_b += om_b * iAf;
         const double Af_b = -om * iAf * om_b;
         const double Bh_b = -oh * oh * oh_b;
@@ -689,65 +754,100 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
 
     // ---- stage C: stencil adjoints per point, ghosts folded onto their source ----
     {
-        double sb[9][N + 2];
-        for (int k = 0; k < 9; ++k)
-            for (int f2 = 0; f2 < N + 2; ++f2) sb[k][f2] = 0.0;
-        // point adjoints before folding: vb[k][field]
-        double vb[9][N + 2];
-        for (int k = 0; k < 9; ++k)
-            for (int f2 = 0; f2 < N + 2; ++f2) vb[k][f2] = 0.0;
-        auto grad_rev = [&](int fld, double gx_b, double gy_b) {
-            vb[1][fld] += gx_b * (1.0 / 3.0);
-            vb[3][fld] -= gx_b * (1.0 / 3.0);
-            vb[5][fld] += gx_b * (1.0 / 12.0) + gy_b * (1.0 / 12.0);
-            vb[6][fld] += -gx_b * (1.0 / 12.0) + gy_b * (1.0 / 12.0);
-            vb[8][fld] += gx_b * (1.0 / 12.0) - gy_b * (1.0 / 12.0);
-            vb[7][fld] += -gx_b * (1.0 / 12.0) - gy_b * (1.0 / 12.0);
-            vb[2][fld] += gy_b * (1.0 / 3.0);
-            vb[4][fld] -= gy_b * (1.0 / 3.0);
-        };
-        for (int p = 0; p < N; ++p) {
-            grad_rev(p, gpx_b[p], gpy_b[p]);
-            for (int k = 1; k < 5; ++k) vb[k][p] += lap_b[p] * (2.0 / 3.0);
-            for (int k = 5; k < 9; ++k) vb[k][p] += lap_b[p] * (1.0 / 6.0);
-            vb[0][p] += lap_b[p] * (-10.0 / 3.0);
-        }
-        grad_rev(N, grx_b, gry_b);
-        grad_rev(N + 1, gsx_b, gsy_b);
-        for (int k = 0; k < 9; ++k) {
-            const int ks = ksrc[k];
-            sb[ks][N] += vb[k][N];
-            sb[ks][N + 1] += vb[k][N + 1];
-            if (wxk[k] < 0 && wyk[k] < 0) {
-                for (int p = 0; p < N; ++p) sb[ks][p] += vb[k][p];
+        // point adjoints of one field from those of its gradient and Laplacian
+        auto points = [&](int fld, double (&vb)[9]) {
+            const double gx_b = fld < N ? gpx_b[fld < N ? fld : 0] : fld == N ? grx_b : gsx_b;
+            const double gy_b = fld < N ? gpy_b[fld < N ? fld : 0] : fld == N ? gry_b : gsy_b;
+            const double lb = fld < N ? lap_b[fld < N ? fld : 0] : 0.0;
+            const double a = gx_b * (1.0 / 12.0), b = gy_b * (1.0 / 12.0), p5 = a + b, p6 = b - a;
+            if (fld < N) {
+                const double l1 = lb * (2.0 / 3.0), l5 = lb * (1.0 / 6.0);
+                vb[0] = lb * (-10.0 / 3.0);
+                vb[1] = fma(4.0, a, l1);
+                vb[3] = fma(-4.0, a, l1);
+                vb[2] = fma(4.0, b, l1);
+                vb[4] = fma(-4.0, b, l1);
+                vb[5] = l5 + p5;
+                vb[7] = l5 - p5;
+                vb[6] = l5 + p6;
+                vb[8] = l5 - p6;
             } else {
-                // ghost phi_p = phi_p(s) + sum_{q != p} cw_pq phi_p(s) phi_q(s)
-                long long sc;
-                int kk2, a1, a2;
-                stencil_source(P, x, y, k, sc, kk2, a1, a2);
-                double ph[N];
-                for (int p = 0; p < N; ++p) ph[p] = B.mac[p * S + sc];
-                for (int p = 0; p < N; ++p) {
-                    sb[ks][p] += vb[k][p];
-                    for (int q = 0; q < N; ++q) {
-                        if (q == p) continue;
-                        double cw = 0.0;
-                        if (wxk[k] >= 0) cw += C.wet[wxk[k]][p][q];
-                        if (wyk[k] >= 0) cw += C.wet[wyk[k]][p][q];
-                        sb[ks][p] += vb[k][p] * cw * ph[q];
-                        sb[ks][q] += vb[k][p] * cw * ph[p];
+                vb[0] = 0.0;
+                vb[1] = 4.0 * a;
+                vb[3] = -vb[1];
+                vb[2] = 4.0 * b;
+                vb[4] = -vb[2];
+                vb[5] = p5;
+                vb[7] = -p5;
+                vb[6] = p6;
+                vb[8] = -p6;
+            }
+        };
+        if (nb.inner) {
+#pragma unroll
+            for (int f2 = 0; f2 < N + 2; ++f2) {
+                double vb[9];
+                points(f2, vb);
+#pragma unroll
+                for (int k = 0; k < 9; ++k) *plane_elem(B.sb, P, k * (N + 2) + f2, (unsigned)c) = vb[k];
+            }
+        } else {
+            double sb[9][N + 2];
+            for (int k = 0; k < 9; ++k)
+                for (int f2 = 0; f2 < N + 2; ++f2) sb[k][f2] = 0.0;
+            for (int f2 = 0; f2 < N + 2; ++f2) {
+                double vb[9];
+                points(f2, vb);
+                for (int k = 0; k < 9; ++k) {
+                    long long sc;
+                    int ks, wx, wy;
+                    stencil_source(P, x, y, k, sc, ks, wx, wy);
+                    sb[ks][f2] += vb[k];
+                    if (f2 < N && (wx >= 0 || wy >= 0)) {
+                        // ghost phi_p = phi_p(s) + sum_{q != p} cw_pq phi_p(s) phi_q(s)
+                        const double php = lbm_ld_ca(B.mac + f2 * S + sc);
+                        for (int q = 0; q < N; ++q) {
+                            if (q == f2) continue;
+                            double cw = 0.0;
+                            if (wx >= 0) cw += C.wet[wx][f2][q];
+                            if (wy >= 0) cw += C.wet[wy][f2][q];
+                            sb[ks][f2] += vb[k] * cw * lbm_ld_ca(B.mac + q * S + sc);
+                            sb[ks][q] += vb[k] * cw * php;
+                        }
                     }
                 }
             }
+            for (int k = 0; k < 9; ++k)
+                for (int f2 = 0; f2 < N + 2; ++f2) B.sb[((long long)k * (N + 2) + f2) * S + c] = sb[k][f2];
         }
-        for (int k = 0; k < 9; ++k)
-            for (int f2 = 0; f2 < N + 2; ++f2) B.sb[((long long)k * (N + 2) + f2) * S + c] = sb[k][f2];
     }
 
     // ---- own stage A + B: eq. 2 sums and eq. H of the cell's own use ----
-    {
-        const double fs_b = rho_b * Rs + mu_b * Ms + lam_b * Ks + cp_b * Cs + psi_b * Dr + chi_b * Pc;
-        const double fl_b = rho_b * Rl + mu_b * Ml + lam_b * Kl + cp_b * Cl - fs_b;
+    if (pure) {
+        // T = rho H / (rho c_p) or (rho H - Lv) / (rho c_p); f_l does not change
+        const double t = T_b * icr, w = -T * t;
+        rhoH_b += t;
+        const double r_b = fma(cp, w, rho_b), c_b = fma(rho, w, cp_b);
+        for (int p = 0; p < N; ++p) {
+            double v = fma(r_b, solid ? C.rho_s[p] : C.rho_l[p],
+                           fma(c_b, solid ? C.cp_s[p] : C.cp_l[p],
+                               fma(mu_b, solid ? C.mu_s[p] : C.mu_l[p], fma(lam_b, solid ? C.lam_s[p] : C.lam_l[p], phi_b[p]))));
+            if (solid) {
+                v = fma(psi_b, C.drho[p], fma(chi_b, C.pcm[p], v));
+            } else {
+                v = fma(-t, P.rhoL[p], v);
+                B.grad[(GS_RHOL + p) * S + c] -= t * phi[p];
+            }
+            phi_b[p] = v;
+            B.grad[((solid ? GS_LAMS : GS_LAML) + p) * S + c] += lam_b * phi[p];
+        }
+    } else {
+        const Mix<N> m = mixture_map<N>(P, phi);
+        const double Ms = mix_sum<N, double>(phi, C.mu_s), Ml = mix_sum<N, double>(phi, C.mu_l);
+        const double Ks = mix_sum<N, double>(phi, C.lam_s), Kl = mix_sum<N, double>(phi, C.lam_l);
+        const double Dr = mix_sum<N, double>(phi, C.drho), Pc = mix_sum<N, double>(phi, C.pcm);
+        const double fs_b = rho_b * m.rs + mu_b * Ms + lam_b * Ks + cp_b * m.cs + psi_b * Dr + chi_b * Pc;
+        const double fl_b = rho_b * m.rl + mu_b * Ml + lam_b * Kl + cp_b * m.cl - fs_b;
         const double Rs_b = rho_b * fs, Rl_b = rho_b * fl, Ms_b = mu_b * fs, Ml_b = mu_b * fl;
         const double Ks_b = lam_b * fs, Kl_b = lam_b * fl, Cs_b = cp_b * fs, Cl_b = cp_b * fl;
         const double Dr_b = psi_b * fs, Pc_b = chi_b * fs;
@@ -763,15 +863,14 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
             B.grad[(GS_LAMS + p) * S + c] += Ks_b * phi[p];
             B.grad[(GS_LAML + p) * S + c] += Kl_b * phi[p];
         }
-        for (int p = 0; p < N; ++p) B.own[p * S + c] = phi_b[p];
-        B.own[N * S + c] = rhoH_b;
     }
+    for (int p = 0; p < N; ++p) B.own[p * S + c] = phi_b[p];
+    B.own[N * S + c] = rhoH_b;
 
     // direct adjoints of the cell's own populations and lagged inputs
     for (int i = 0; i < 9; ++i) {
         B.apop[pidx(P, 0, i, c)] = f_b[i];
         B.apop[pidx(P, N + 1, i, c)] = h_b[i];
-        for (int p = 0; p < N; ++p) B.apop[pidx(P, 1 + p, i, c)] = g_b[p][i];
     }
     B.aaux[aux_mdot() * S + c] = 0.0;
     B.aaux[aux_Q() * S + c] = 0.0;
@@ -784,7 +883,7 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const KParams P, const Ad
 // is ill-conditioned where little phase-changing material is present: the mushy band
 // of eq. H is Lv wide, and Lv -> 0 there; weighted by phi_pcm it is not.)
 template <int N, bool SEED>
-__global__ void __launch_bounds__(128) adj_moments_kernel(const KParams P, const AdjBufs B)
+__global__ void __launch_bounds__(ADJ_NT) adj_moments_kernel(const KParams P, const AdjBufs B)
 {
     const long long S = P.S;
     const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -797,77 +896,89 @@ __global__ void __launch_bounds__(128) adj_moments_kernel(const KParams P, const
     if (!SEED) {
         for (int p = 0; p < N; ++p) phi_b[p] = B.own[p * S + c];
         rhoH_b = B.own[N * S + c];
+#pragma unroll
         for (int k = 0; k < 9; ++k) {
-            // the user x = y - c_k used y as its stencil point k
+            // the user x = y - c_k used y as its stencil point k; beyond a side there is none (its
+            // index is then y's own)
             int ux_ = x - cx(k), uy_ = y - cy(k);
+            bool user = true;
             if (ux_ < 0 || ux_ >= P.nx) {
-                if (!xper) continue;
-                ux_ = wrap_index(ux_, P.nx);
+                if (xper) ux_ = wrap_index(ux_, P.nx);
+                else user = false;
             }
             if (uy_ < 0 || uy_ >= P.ny) {
-                if (!yper) continue;
-                uy_ = wrap_index(uy_, P.ny);
+                if (yper) uy_ = wrap_index(uy_, P.ny);
+                else user = false;
             }
-            const long long uc = (long long)uy_ * P.nx + ux_;
-            for (int p = 0; p < N; ++p) phi_b[p] += B.sb[((long long)k * (N + 2) + p) * S + uc];
-            rho_b += B.sb[((long long)k * (N + 2) + N) * S + uc];
-            psi_b += B.sb[((long long)k * (N + 2) + N + 1) * S + uc];
+            const unsigned uc = user ? (unsigned)uy_ * (unsigned)P.nx + (unsigned)ux_ : (unsigned)c;
+            if (!user) continue;
+#pragma unroll
+            for (int p = 0; p < N; ++p) phi_b[p] += lbm_ld_ca(plane_elem(B.sb, P, k * (N + 2) + p, uc));
+            rho_b += lbm_ld_ca(plane_elem(B.sb, P, k * (N + 2) + N, uc));
+            psi_b += lbm_ld_ca(plane_elem(B.sb, P, k * (N + 2) + N + 1, uc));
         }
     }
-    // recompute the moments and eq. H of y
-    double g[N][9], h[9];
-    for (int i = 0; i < 9; ++i) {
-        h[i] = B.pin[pidx(P, N + 1, i, c)];
-        for (int p = 0; p < N; ++p) g[p][i] = B.pin[pidx(P, 1 + p, i, c)];
+    // eq. H of y, from its moments (mac_kernel; the loss seed has none and adds them up here)
+    const double mdm = B.ain[aux_mdot() * S + c];
+    double phi[N], rhoH, iden = 1.0;
+    if (mdm != 0.0) iden = 1.0 / fma(-0.5, mdm, 1.0);
+    if (SEED) {
+        for (int p = 0; p < N; ++p) {
+            double sg = 0.0;
+            for (int i = 0; i < 9; ++i) sg += B.pin[pidx(P, 1 + p, i, c)];
+            phi[p] = sg * iden;
+        }
+        double sh = 0.0;
+        for (int i = 0; i < 9; ++i) sh += B.pin[pidx(P, N + 1, i, c)];
+        rhoH = fma(0.5, B.ain[aux_Q() * S + c], sh);
+    } else {
+        for (int p = 0; p < N; ++p) phi[p] = B.mac[p * S + c];
+        rhoH = B.mac[(N + 2) * S + c];
     }
-    const double mdm = B.ain[aux_mdot() * S + c], Qm = B.ain[aux_Q() * S + c];
-    const double iden = 1.0 / (1.0 - 0.5 * mdm);
-    double phi[N];
-    for (int p = 0; p < N; ++p) {
-        double sg = 0.0;
-        for (int i = 0; i < 9; ++i) sg += g[p][i];
-        phi[p] = sg * iden;
-    }
-    double sh = 0.0;
-    for (int i = 0; i < 9; ++i) sh += h[i];
-    const double rhoH = fma(0.5, Qm, sh);
-    const Mix<N> m = mixture_map<N>(P, phi);
-    double fl, T;
-    enthalpy_map<N, false>(P, m, rhoH, fl, T);
+    double fl;
+    const int branch = eqh_branch<N>(P, phi, rhoH, fl);
     const double fs = 1.0 - fl;
-    const double Rs = mix_sum<N, double>(phi, C.rho_s), Rl = mix_sum<N, double>(phi, C.rho_l);
-    const double Dr = mix_sum<N, double>(phi, C.drho);
     double fl_b = 0.0;
     if (SEED) {
         // q = phi_pcm f_l, the liquid fraction of the phase-changing material
         // (phi_pcm = sum_p phi_p over the phases with L_p > 0)
         const double Pc = mix_sum<N, double>(phi, C.pcm);
-        const double w = B.weight ? B.weight[c] : 1.0;
+        const double w = B.weight ? lbm_ld_ca(B.weight + c) : 1.0;
         const double d = Pc * fl - B.fl_target[c];
         const double q_b = 2.0 * w * d;
         fl_b = q_b * Pc;
         for (int p = 0; p < N; ++p) phi_b[p] += q_b * fl * C.pcm[p];
         B.grad[(long long)GS_LOSS * S + c] = w * d * d;
     }
-    // rho = fs Rs + fl Rl, psi = fs Dr
-    const double fs_b = rho_b * Rs + psi_b * Dr;
-    fl_b += rho_b * Rl - fs_b;
-    const double Rs_b = rho_b * fs, Rl_b = rho_b * fl, Dr_b = psi_b * fs;
-    double rs_b = 0, rl_b = 0, cs_b = 0, cl_b = 0, Lv_b = 0;
-    map_reverse<N>(P, m, rhoH, fl_b, 0.0, rs_b, rl_b, cs_b, cl_b, Lv_b, rhoH_b);
+    // rho = fs Rs + fl Rl, psi = fs Dr; where f_l is 1 or 0 it does not change
+    if (branch == EQH_LIQUID) {
+        for (int p = 0; p < N; ++p) phi_b[p] = fma(rho_b, C.rho_l[p], phi_b[p]);
+    } else if (branch == EQH_SOLID) {
+        for (int p = 0; p < N; ++p) phi_b[p] = fma(rho_b, C.rho_s[p], fma(psi_b, C.drho[p], phi_b[p]));
+    } else {
+        const Mix<N> m = mixture_map<N>(P, phi);
+        const double Dr = mix_sum<N, double>(phi, C.drho);
+        const double fs_b = rho_b * m.rs + psi_b * Dr;
+        fl_b += rho_b * m.rl - fs_b;
+        const double Rs_b = rho_b * fs, Rl_b = rho_b * fl, Dr_b = psi_b * fs;
+        double rs_b = 0, rl_b = 0, cs_b = 0, cl_b = 0, Lv_b = 0;
+        map_reverse<N>(P, m, rhoH, fl_b, 0.0, rs_b, rl_b, cs_b, cl_b, Lv_b, rhoH_b);
+        for (int p = 0; p < N; ++p) {
+            phi_b[p] += Rs_b * C.rho_s[p] + Rl_b * C.rho_l[p] + Dr_b * C.drho[p];
+            phi_b[p] += rs_b * P.d.rho_s[p] + rl_b * P.d.rho_l[p] + cs_b * P.d.cp_s[p] + cl_b * P.d.cp_l[p] +
+                        Lv_b * P.rhoL[p];
+            B.grad[(GS_RHOL + p) * S + c] += Lv_b * phi[p];
+        }
+    }
     double mdm_b = 0.0;
     for (int p = 0; p < N; ++p) {
-        phi_b[p] += Rs_b * C.rho_s[p] + Rl_b * C.rho_l[p] + Dr_b * C.drho[p];
-        phi_b[p] += rs_b * P.d.rho_s[p] + rl_b * P.d.rho_l[p] + cs_b * P.d.cp_s[p] + cl_b * P.d.cp_l[p] +
-                    Lv_b * P.rhoL[p];
-        B.grad[(GS_RHOL + p) * S + c] += Lv_b * phi[p];
         // phi_p = (sum_i g_ip) / (1 - mdot'/2)
         const double gb = phi_b[p] * iden;
         for (int i = 0; i < 9; ++i) {
             const long long k = pidx(P, 1 + p, i, c);
             B.apop[k] = SEED ? gb : B.apop[k] + gb;
         }
-        mdm_b += phi_b[p] * phi[p] * 0.5 * iden;
+        mdm_b = fma(0.5 * gb, phi[p], mdm_b);
     }
     // rho H = sum_i h_i + Q'/2
     for (int i = 0; i < 9; ++i) {

@@ -145,7 +145,7 @@ extern "C" int lbm_adjoint_fl_loss(lbm_handle* h, const double* phi0, const doub
     ADJ_TRY(h, ck.alloc(std::max<long>(nck, 1) * set_bytes));
     ADJ_TRY(h, seg.alloc((size_t)K * set_bytes));
     ADJ_TRY(h, abar.alloc(2 * set_bytes));
-    ADJ_TRY(h, mac.alloc((size_t)(N + 2) * plane));
+    ADJ_TRY(h, mac.alloc((size_t)(N + 3) * plane));
     ADJ_TRY(h, own.alloc((size_t)(N + 1) * plane));
     ADJ_TRY(h, sb.alloc((size_t)9 * (N + 2) * plane));
     ADJ_TRY(h, grad.alloc((size_t)(GS_COUNT + 1) * plane));

@@ -152,15 +152,15 @@ __device__ __forceinline__ V phi_sum(const V (&phi)[N], const C (&a)[MAXN])
     return v;
 }
 
-// eq. H for one cell: the liquid fraction, as the FP64 map gives it.  A screen in FP32 decides
-// the cells whose rho H lies above the liquidus value Al, or (with phase-changing material
-// present) below the solidus value As, by more than 1e-5 of the magnitudes involved: at least
-// ten times the rounding of As and Al from leading parts.  Only the other cells (the mushy
-// band, values near a threshold, phase-changing material below FP32 range, values that are not
-// finite) run the FP64 map.  Where the solidus value can lie above the liquidus value
-// (P.ordered = 0), a liquid cell has to clear both, as in the map.
+// The FP32 screen of eq. H for one cell: 1 (liquid) where rho H lies above the liquidus value Al, 0
+// (solid) where phase-changing material is present and rho H lies below the solidus value As, by
+// more than 1e-5 of the magnitudes involved: at least ten times the rounding of As and Al from
+// leading parts; -1 where it does not decide (the mushy band, values near a threshold,
+// phase-changing material below FP32 range, values that are not finite).  Where the solidus
+// value can lie above the liquidus value (P.ordered = 0), a liquid cell has to clear both, as
+// in the map.
 template <int N, class V>
-__device__ __forceinline__ V liquid_fraction(const KParams& P, const V (&phi)[N], V rhoH)
+__device__ __forceinline__ int eqh_screen(const KParams& P, const V (&phi)[N], V rhoH)
 {
     const Coef<float>& C = P.f;
     float ph[N];
@@ -177,7 +177,7 @@ __device__ __forceinline__ V liquid_fraction(const KParams& P, const V (&phi)[N]
     const float Ac = __fmul_rn(__fmul_rn(rl, cl), C.T_liq), Al = __fadd_rn(Ac, Lv);
     const float tol = __fmaf_rn(1e-5f, __fadd_rn(__fadd_rn(fabsf(Ac), fabsf(Lv)), fabsf(h)), 1e-30f);
     const bool above = h > __fadd_rn(Al, tol);
-    if (above && P.ordered) return V(1.0f);
+    if (above && P.ordered) return 1;
     float rs = __fmul_rn(ph[0], C.rho_s[0]), cs = __fmul_rn(ph[0], C.cp_s[0]);
 #pragma unroll
     for (int p = 1; p < N; ++p) {
@@ -186,8 +186,19 @@ __device__ __forceinline__ V liquid_fraction(const KParams& P, const V (&phi)[N]
     }
     const float As = __fmul_rn(__fmul_rn(rs, cs), C.T_sol);
     const float tols = __fmaf_rn(1e-5f, fabsf(As), tol);
-    if (above && h > __fadd_rn(As, tols)) return V(1.0f);
-    if (Lv > 0.0f && h < __fsub_rn(As, tols)) return V(0.0f);
+    if (above && h > __fadd_rn(As, tols)) return 1;
+    if (Lv > 0.0f && h < __fsub_rn(As, tols)) return 0;
+    return -1;
+}
+
+// eq. H for one cell: the liquid fraction, as the FP64 map gives it (the map itself runs only where
+// the screen does not decide).
+template <int N, class V>
+__device__ __forceinline__ V liquid_fraction(const KParams& P, const V (&phi)[N], V rhoH)
+{
+    const int sure = eqh_screen<N>(P, phi, rhoH);
+    if (sure > 0) return V(1.0f);
+    if (sure == 0) return V(0.0f);
     double phd[N], fl, T;
 #pragma unroll
     for (int p = 0; p < N; ++p) phd[p] = (double)phi[p];

@@ -238,24 +238,24 @@ cudaError_t launch_batch_staged(const BatchTable& T, const StageMaps* maps, int 
 template <int N>
 cudaError_t launch_adj_mac(const KParams& P, const double* pin, const double* ain, double* mac, cudaStream_t st)
 {
-    const long long blocks = std::min<long long>((P.S + 255) / 256, 65535);
-    mac_kernel<N><<<(int)blocks, 256, 0, st>>>(P, pin, ain, mac);
+    const long long blocks = std::min<long long>((P.S + ADJ_NT - 1) / ADJ_NT, 1 << 20);
+    mac_kernel<N><<<(int)blocks, ADJ_NT, 0, st>>>(P, pin, ain, mac);
     return cudaGetLastError();
 }
 
 template <int N>
 cudaError_t launch_adj_cell(const KParams& P, const AdjBufs& B, cudaStream_t st)
 {
-    adj_cell_kernel<N><<<(unsigned)((P.S + 127) / 128), 128, 0, st>>>(P, B);
+    adj_cell_kernel<N><<<(unsigned)((P.S + ADJ_NT - 1) / ADJ_NT), ADJ_NT, 0, st>>>(P, B);
     return cudaGetLastError();
 }
 
 template <int N>
 cudaError_t launch_adj_moments(const KParams& P, const AdjBufs& B, bool seed, cudaStream_t st)
 {
-    const unsigned blocks = (unsigned)((P.S + 127) / 128);
-    if (seed) adj_moments_kernel<N, true><<<blocks, 128, 0, st>>>(P, B);
-    else adj_moments_kernel<N, false><<<blocks, 128, 0, st>>>(P, B);
+    const unsigned blocks = (unsigned)((P.S + ADJ_NT - 1) / ADJ_NT);
+    if (seed) adj_moments_kernel<N, true><<<blocks, ADJ_NT, 0, st>>>(P, B);
+    else adj_moments_kernel<N, false><<<blocks, ADJ_NT, 0, st>>>(P, B);
     return cudaGetLastError();
 }
 

@@ -190,15 +190,15 @@ __device__ __forceinline__ void cell_moments(const KParams& P, const L& ld, type
     fl = liquid_fraction<N>(P, phi, rhoH);
 }
 
-// phi_p, rho and psi of a cell (what its neighbours' stencils read).
+// phi_p, rho and psi of a cell (what its neighbours' stencils read), and rho H.
 template <int N, class Pr>
 __device__ __forceinline__ void halo_moments(const KParams& P, const PopView<Pr>& pin,
                                              const typename Pr::TA* __restrict__ ain, unsigned c,
                                              val_t<typename Pr::R> (&phi)[N], val_t<typename Pr::R>& rho,
-                                             val_t<typename Pr::R>& psi)
+                                             val_t<typename Pr::R>& psi, val_t<typename Pr::R>& rhoH)
 {
     const GlobalLoader<Pr> ld{P, pin, ain};
-    val_t<typename Pr::R> rhoH, fl;
+    val_t<typename Pr::R> fl;
     cell_moments<N, Pr>(P, ld, c, phi, rhoH, fl);
     mix_rho_psi<N>(P, phi, fl, rho, psi);
 }
