@@ -24,7 +24,7 @@
 // coefficients alone, its moments come from mac_kernel's planes (so the cell kernel reads no
 // phase-field population), its quotients from one reciprocal, and the stencil adjoints of a cell away
 // from the sides go straight to their planes.  256 x 256, N = 4, us per launch, before and after:
-// mac 18 / 12, cell 306 / 272, moments 59 / 40.
+// mac 18 / 13, cell 306 / 208, moments 59 / 41.
 //
 // Parameter gradients accumulate per cell in FP64 planes (slot layout below) and are
 // reduced once at the end, in a fixed order.
@@ -273,14 +273,51 @@ __device__ __forceinline__ void stencil_source(const KParams& P, int x, int y, i
     ksrc = dir_of(dx, dy);
 }
 
+// Threads of adj_cell_kernel: the cells at the sides first, in warps of their own, then the others.
+// A cell at a side takes several times the instructions of any other (push targets, wrapped and
+// ghost stencil points); in lattice order every row has two of them, and at 256 x 256 a quarter of
+// all warps ran both paths (272 us a launch; now 208).
+__host__ __device__ inline long long adj_side_threads(int nx, int ny)
+{
+    return ((2LL * nx + 2LL * (ny - 2)) + 31) / 32 * 32;
+}
+__host__ __device__ inline long long adj_cell_threads(int nx, int ny)
+{
+    return adj_side_threads(nx, ny) + (long long)(nx - 2) * (ny - 2);
+}
+// The cell of thread t; false for none.
+__device__ __forceinline__ bool adj_cell_of(const KParams& P, long long t, int& x, int& y)
+{
+    const int nx = P.nx, ny = P.ny;
+    const long long side = adj_side_threads(nx, ny);
+    if (t >= side) {
+        t -= side;
+        if (t >= (long long)(nx - 2) * (ny - 2)) return false;
+        x = 1 + (int)(t % (nx - 2));
+        y = 1 + (int)(t / (nx - 2));
+        return true;
+    }
+    int k = (int)t;
+    if (k < 2 * nx) {
+        x = k % nx;
+        y = k < nx ? 0 : ny - 1;
+        return true;
+    }
+    k -= 2 * nx;
+    if (k >= 2 * (ny - 2)) return false;
+    x = k & 1 ? nx - 1 : 0;
+    y = 1 + (k >> 1);
+    return true;
+}
+
 // The adjoint of one cell's step (see the file comment).
 template <int N>
 __global__ void __launch_bounds__(ADJ_NT) adj_cell_kernel(const KParams P, const AdjBufs B)
 {
     const long long S = P.S;
-    const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (c >= S) return;
-    const int x = (int)(c % P.nx), y = (int)(c / P.nx);
+    int x, y;
+    if (!adj_cell_of(P, blockIdx.x * (long long)blockDim.x + threadIdx.x, x, y)) return;
+    const long long c = (long long)y * P.nx + x;
     const Coef<double>& C = P.d;
 
     const Neighbours nb(P, x, y);

@@ -246,7 +246,7 @@ cudaError_t launch_adj_mac(const KParams& P, const double* pin, const double* ai
 template <int N>
 cudaError_t launch_adj_cell(const KParams& P, const AdjBufs& B, cudaStream_t st)
 {
-    adj_cell_kernel<N><<<(unsigned)((P.S + ADJ_NT - 1) / ADJ_NT), ADJ_NT, 0, st>>>(P, B);
+    adj_cell_kernel<N><<<(unsigned)((adj_cell_threads(P.nx, P.ny) + ADJ_NT - 1) / ADJ_NT), ADJ_NT, 0, st>>>(P, B);
     return cudaGetLastError();
 }
 
