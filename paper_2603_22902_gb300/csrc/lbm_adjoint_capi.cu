@@ -142,7 +142,7 @@ extern "C" int lbm_adjoint_fl_loss(lbm_handle* h, const double* phi0, const doub
 
     // working memory: checkpoints, one recomputed segment, adjoint sets and planes
     DevBuf ck, seg, abar, mac, own, sb, grad, part, sums;
-    ADJ_TRY(h, ck.alloc(std::max<long>(nck, 1) * set_bytes));
+    ADJ_TRY(h, ck.alloc(std::max<long>(nck - 1, 1) * set_bytes));
     ADJ_TRY(h, seg.alloc((size_t)K * set_bytes));
     ADJ_TRY(h, abar.alloc(2 * set_bytes));
     ADJ_TRY(h, mac.alloc((size_t)(N + 3) * plane));
@@ -163,8 +163,28 @@ extern "C" int lbm_adjoint_fl_loss(lbm_handle* h, const double* phi0, const doub
     h->cur = 0;
     h->ready = true;
     h->steps = 0;
+    // The steps of the last segment write their states where the reverse sweep reads them, so that it is
+    // not recomputed (nsteps 20, K = 5: 32 steps instead of 36).
+    const long last0 = nck > 0 ? (nck - 1) * (long)K : 0;
+    auto seg_state = [&](long j) { return seg.as<char>() + (size_t)j * set_bytes; };
     for (long n = 0; n < nsteps; ++n) {
         const int a = h->cur, b = a ^ 1;
+        if (n == last0) {
+            ADJ_TRY(h, cudaMemcpyAsync(pop_of(seg_state(0)), h->pop[a], h->pop_bytes, cudaMemcpyDeviceToDevice, st));
+            ADJ_TRY(h, cudaMemcpyAsync(aux_of(seg_state(0)), h->aux[a], h->aux_bytes, cudaMemcpyDeviceToDevice, st));
+        }
+        if (n >= last0) {
+            const bool final = n == nsteps - 1;
+            char *from = seg_state(n - last0), *to = seg_state(final ? n - last0 : n - last0 + 1);
+            e = dispatch(N, LBM_FP64, [&](auto nn, auto pr) {
+                return launch_step<decltype(nn)::value, decltype(pr)>(P, pop_of(from), final ? h->pop[b] : pop_of(to), aux_of(from),
+                                                                      final ? h->aux[b] : aux_of(to), lbm_step_tile(h), st);
+            });
+            if (e != cudaSuccess) return acuda(h, e, "step kernel");
+            if (final) h->cur = b;
+            h->steps++;
+            continue;
+        }
         if (n % K == 0) {
             char* c0 = ck.as<char>() + (size_t)(n / K) * set_bytes;
             ADJ_TRY(h, cudaMemcpyAsync(pop_of(c0), h->pop[a], h->pop_bytes, cudaMemcpyDeviceToDevice, st));
@@ -199,12 +219,12 @@ extern "C" int lbm_adjoint_fl_loss(lbm_handle* h, const double* phi0, const doub
     // ---- reverse sweep: per segment, recompute its states, then step back ----
     for (long sgi = nck - 1; sgi >= 0; --sgi) {
         const long n0 = sgi * K, n1 = std::min<long>(nsteps, n0 + K);
-        char* s0 = seg.as<char>();
-        const char* c0 = ck.as<char>() + (size_t)sgi * set_bytes;
-        ADJ_TRY(h, cudaMemcpyAsync(s0, c0, set_bytes, cudaMemcpyDeviceToDevice, st));
-        for (long j = 1; j < n1 - n0; ++j) {
-            char* sa = seg.as<char>() + (size_t)(j - 1) * set_bytes;
-            char* sbn = seg.as<char>() + (size_t)j * set_bytes;
+        if (sgi < nck - 1) {
+            const char* c0 = ck.as<char>() + (size_t)sgi * set_bytes;
+            ADJ_TRY(h, cudaMemcpyAsync(seg_state(0), c0, set_bytes, cudaMemcpyDeviceToDevice, st));
+        }
+        for (long j = 1; sgi < nck - 1 && j < n1 - n0; ++j) {
+            char *sa = seg_state(j - 1), *sbn = seg_state(j);
             e = dispatch(N, LBM_FP64, [&](auto nn, auto pr) {
                 return launch_step<decltype(nn)::value, decltype(pr)>(P, pop_of(sa), pop_of(sbn), aux_of(sa), aux_of(sbn),
                                                                       lbm_step_tile(h), st);
@@ -212,7 +232,7 @@ extern "C" int lbm_adjoint_fl_loss(lbm_handle* h, const double* phi0, const doub
             if (e != cudaSuccess) return acuda(h, e, "recompute step kernel");
         }
         for (long n = n1 - 1; n >= n0; --n) {
-            char* sa = seg.as<char>() + (size_t)(n - n0) * set_bytes;
+            char* sa = seg_state(n - n0);
             B.pin = (const double*)pop_of(sa);
             B.ain = (const double*)aux_of(sa);
             B.bpop = (const double*)pop_of(abuf[ia]);
