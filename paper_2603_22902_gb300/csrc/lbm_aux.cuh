@@ -14,6 +14,32 @@ namespace lbm {
 template <class R>
 using init_t = typename std::conditional<std::is_same<R, double>::value, double, df64>::type;
 
+// An FP64 input of the initial state as the arithmetic type.  For double words: the pair of
+// df64(double) (x rounded to FP32, and the rest rounded to FP32; of two equally near x the one
+// further from zero), put together with integer instructions.  The four FP64 instructions of
+// the conversion occupy a scheduler's share of the FP64 unit for 64 cycles each: the N + 3
+// inputs held that unit for 43 of the kernel's 78 us at 1024^2, N = 3, FP16 storage.  Only values
+// so small or so large that a part would leave FP32's normal range are converted there.
+template <class I>
+__device__ __forceinline__ I init_input(double x)
+{
+    if constexpr (std::is_same<I, df64>::value) {
+        constexpr int ONE = 0x00100000;                     // one of a double's exponent, in its upper word
+        const int h = __double2hiint(x), l = __double2loint(x);
+        if ((unsigned)((h & 0x7ff00000) - (1023 - 70) * ONE) < 196u * ONE) {
+            const unsigned bl = (unsigned)l + 0x10000000u;  // half of the last bit that hi keeps
+            const int bh = h + (bl < 0x10000000u);
+            const unsigned hi = ((unsigned)((bh & 0x7fffffff) - 896 * ONE) << 3) | (bl >> 29);
+            const unsigned unit = (unsigned)((h & 0x7ff00000) - 948 * ONE) << 3;   // 2^(exponent - 52)
+            const float lo = (float)((int)(bl & 0x1fffffffu) - 0x10000000);
+            const unsigned sign = (unsigned)h & 0x80000000u;
+            return df64(__uint_as_float(hi | sign), lo * __uint_as_float(unit | sign));
+        }
+        if (((h << 1) | l) == 0) return df64(__int_as_float(h), 0.0f);   // 0 and -0
+    }
+    return I(x);
+}
+
 // A value of the initial state as the policy's arithmetic type (rounded once).
 template <class R, class I>
 __device__ __forceinline__ R init_value(I v)
@@ -89,11 +115,14 @@ __device__ __forceinline__ bool init_macro_decided(const KParams& P, const df64 
 // converted on the same unit) the kernel was bound by the 2-lane FP64 pipe for every policy:
 // 1676 us at 2048^2, N = 2, FP16 storage, against 95 us for its bytes.  The policies that
 // store FP32 or less, and double words, now work in double words (an FP32 result is the
-// double word rounded once): 250 us there.  FP64 decides the cells that eq. H does not decide
-// by a margin.
+// double word rounded once): 160 us there.  FP64 decides the cells that eq. H does not decide
+// by a margin.  What bounds it now is the number of its instructions (1720 per 32 cells at N = 3,
+// 64 % of the issue slots).  Three blocks to an SM where 16-bit values are stored (a pass over 2048^2
+// with 20 steps: 4619 us with two, 4578 with three); two for the wider types, whose three-phase kernel
+// spills at 80 registers (1024^2, N = 3, FP32: 2284 us with two, 2316 with three).
 // Populations come in opposite pairs, whose even and odd parts in c_i . u are shared.
 template <int N, class Pr>
-__global__ void __launch_bounds__(256, 2) init_kernel(const KParams P, const double* __restrict__ phi_in, const double* __restrict__ T_in,
+__global__ void __launch_bounds__(256, sizeof(typename Pr::TM) == 2 ? 3 : 2) init_kernel(const KParams P, const double* __restrict__ phi_in, const double* __restrict__ T_in,
                             const double* __restrict__ ux_in, const double* __restrict__ uy_in,
                             void* __restrict__ pop_base, typename Pr::TA* __restrict__ aux)
 {
@@ -108,10 +137,11 @@ __global__ void __launch_bounds__(256, 2) init_kernel(const KParams P, const dou
 #pragma unroll
         for (int p = 0; p < N; ++p) phd[p] = LBM_LD(P, phi_in, p * S + c, N * S, 40);
         const double T0 = LBM_LD(P, T_in, c, S, 43);
-        const I ux = ux_in ? I(LBM_LD(P, ux_in, c, S, 41)) : I(0.0), uy = uy_in ? I(LBM_LD(P, uy_in, c, S, 42)) : I(0.0);
-        I phi[N], rhoH, T = I(T0), rho, cp, psi;
+        const I ux = ux_in ? init_input<I>(LBM_LD(P, ux_in, c, S, 41)) : I(0.0),
+                uy = uy_in ? init_input<I>(LBM_LD(P, uy_in, c, S, 42)) : I(0.0);
+        I phi[N], rhoH, T = init_input<I>(T0), rho, cp, psi;
 #pragma unroll
-        for (int p = 0; p < N; ++p) phi[p] = I(phd[p]);
+        for (int p = 0; p < N; ++p) phi[p] = init_input<I>(phd[p]);
         bool decided = false;
         if constexpr (!std::is_same<I, double>::value) decided = init_macro_decided<N>(P, phi, T, rhoH, rho, cp, psi);
         if (!decided) {
@@ -152,8 +182,14 @@ __global__ void __launch_bounds__(256, 2) init_kernel(const KParams P, const dou
 #pragma unroll
             for (int p = 0; p < N; ++p) {
                 const I wp = w * phi[p];
-                put(G{}, 1 + p, i, rfma(wp, odd, wp));
-                put(G{}, 1 + p, j, rfma(-wp, odd, wp));
+                if constexpr (std::is_same<I, double>::value) {
+                    put(G{}, 1 + p, i, rfma(wp, odd, wp));
+                    put(G{}, 1 + p, j, rfma(-wp, odd, wp));
+                } else {   // the product once: the same values
+                    const I t = wp * odd;
+                    put(G{}, 1 + p, i, t + wp);
+                    put(G{}, 1 + p, j, wp - t);
+                }
             }
         }
         LBM_ST(P, aux, aux_mdot() * S + c, P.aux_elems, 47, (TA)0.0);

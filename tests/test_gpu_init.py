@@ -71,3 +71,30 @@ def test_initial_state_is_the_fp64_one(prec, kind, size):
         scale = np.abs(a).max(axis=tuple(range(1, a.ndim)), keepdims=True)
         floor = 2.0 ** -24 * np.array([1 / 4096.0] + [1.0] * (case.N + 1))[:, None, None] if prec == "fp16s" and k == 0 else 0.0
         assert np.all(np.abs(a - b) <= unit * np.abs(a) + 64 * 2.0 ** -48 * scale + floor), (k, np.abs(a - b).max())
+
+
+@pytest.mark.parametrize("prec", ["df64", "fp32"])
+def test_inputs_of_every_magnitude_and_at_rounding_ties(prec):
+    """(phi_0 u)' with phi_0 = 1 is the input u: zeros of either sign, the powers of two around the range that
+    integer instructions convert (2^-70 ... 2^126 is beyond any velocity; up to 2^-4 here), values half-way between
+    two FP32 numbers, one bit beside them, and values whose rounding carries into the exponent."""
+    case = _case("sharp", 40, 33)
+    S = case.nx * case.ny
+    case.phi = np.zeros_like(case.phi)
+    case.phi[0] = 1.0
+    e = np.arange(S) % 140 - 143                             # 2^-143 ... 2^-4
+    one = np.float64(1.0).view(np.int64)
+    low = np.array([0, 1, 0x0fffffff, 0x10000000, 0x10000001, 0x1fffffff, 0x30000000, 0xfffffffffffff, 0xffffff0000000])
+    m = (one + low[np.arange(S) % len(low)]).view(np.float64)
+    u = np.ldexp(m, e) * np.where(np.arange(S) % 2, -1.0, 1.0)
+    u[::50] = 0.0
+    u[1::50] = -0.0
+    case.ux, case.uy = u.reshape(case.ny, case.nx), u[::-1].reshape(case.ny, case.nx).copy()
+    from paper_2603_22902_gb300 import lbm as L
+    _, aux = _state(L, case, prec)
+    # the pair of words holds the input to 2^-48, the product with 1 adds 4 2^-48; FP32 rounds once; words below
+    # 2^-126 are multiples of 2^-149
+    unit = {"df64": 5 * 2.0 ** -48, "fp32": 2.0 ** -24 * (1.0 + 2.0 ** -9)}[prec]
+    for got, want in ((aux[3], case.ux), (aux[3 + case.N], case.uy)):
+        want = want.reshape(-1)
+        assert np.all(np.abs(got - want) <= unit * np.abs(want) + 2.0 ** -147), np.abs(got - want).max()
