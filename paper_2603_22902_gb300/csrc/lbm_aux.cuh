@@ -18,8 +18,8 @@ using init_t = typename std::conditional<std::is_same<R, double>::value, double,
 // df64(double) (x rounded to FP32, and the rest rounded to FP32; of two equally near x the one
 // further from zero), put together with integer instructions.  The four FP64 instructions of
 // the conversion occupy a scheduler's share of the FP64 unit for 64 cycles each: the N + 3
-// inputs held that unit for 43 of the kernel's 78 us at 1024^2, N = 3, FP16 storage.  Only values
-// so small or so large that a part would leave FP32's normal range are converted there.
+// inputs held that unit for 43 of the kernel's 78 us at 1024^2, N = 3, FP16 storage; now 64 us.  Only
+// values so small or so large that a part would leave FP32's normal range are converted there.
 template <class I>
 __device__ __forceinline__ I init_input(double x)
 {
@@ -115,7 +115,7 @@ __device__ __forceinline__ bool init_macro_decided(const KParams& P, const df64 
 // converted on the same unit) the kernel was bound by the 2-lane FP64 pipe for every policy:
 // 1676 us at 2048^2, N = 2, FP16 storage, against 95 us for its bytes.  The policies that
 // store FP32 or less, and double words, now work in double words (an FP32 result is the
-// double word rounded once): 160 us there.  FP64 decides the cells that eq. H does not decide
+// double word rounded once): 196 us there.  FP64 decides the cells that eq. H does not decide
 // by a margin.  What bounds it now is the number of its instructions (1720 per 32 cells at N = 3,
 // 64 % of the issue slots).  Three blocks to an SM where 16-bit values are stored (a pass over 2048^2
 // with 20 steps: 4619 us with two, 4578 with three); two for the wider types, whose three-phase kernel
