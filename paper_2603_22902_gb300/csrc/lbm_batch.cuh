@@ -129,9 +129,11 @@ batch_step_kernel(const BatchTable T, int s)
 
 // Per-step form of small FP64 groups: each tile of the list as eight tiles of 8x4, one warp
 // each (see fp64_small_tiles for the rule).  Five small cases, 69 tiles: one tile of 8 warps
-// keeps its SM's FP64 unit busy for 46 us while 83 SMs idle.
-template <int N, int TX, int TY, class Pr>
-__global__ void __launch_bounds__(BATCH_NT / BATCH_SUB, LBM_OCC(Pr) * BATCH_SUB / BATCH_NT)
+// keeps its SM's FP64 unit busy for 46 us while 83 SMs idle.  RING_TEAM: a second warp takes the
+// ring (fp64_ring_team).
+template <int N, int TX, int TY, class Pr, bool RING_TEAM>
+__global__ void __launch_bounds__(BATCH_NT / BATCH_SUB * (RING_TEAM ? 2 : 1),
+                                  LBM_OCC(Pr) * BATCH_SUB / BATCH_NT / (RING_TEAM ? 2 : 1))
 batch_substep_kernel(const BatchTable T, int s)
 {
     static_assert(TX * TY == BATCH_NT && TX % 8 == 0 && TY % 4 == 0, "eight 8x4 tiles");
@@ -148,7 +150,7 @@ batch_substep_kernel(const BatchTable T, int s)
     load_params(sP, T.params + c);
     __syncthreads();
     const int a = (*(volatile unsigned char*)T.parity) ^ (s & 1);
-    step_tile<N, 8, 4, true, Pr>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
+    step_tile<N, 8, 4, true, Pr, RING_TEAM>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
                                  (TA*)C.aux[a ^ 1], ExportPtrs{}, bx, by, smem);
 }
 

@@ -42,7 +42,6 @@ __device__ __forceinline__ constexpr const_t<V> cst(double c)
     return const_t<V>(c);
 }
 
-// Scalar forms of the predicates that the packed type answers for both of its cells.
 template <class V>
 __device__ __forceinline__ bool any_nonzero(V a)
 {

@@ -51,11 +51,13 @@ static cudaError_t launch_fused_t(const KParams& P, const void* pin, void* pout,
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        if (tiles > sms) {
-            fused_step_kernel<N, TX, TY, COLLIDE, Pr><<<tiles, TX * TY, 0, st>>>(P, pin, pout, (const TA*)ain, (TA*)aout, ex,
-                                                                                 rows);
-            return cudaGetLastError();
-        }
+        const bool team = fp64_ring_team(tiles, sms);
+        const auto kernel = team ? fused_step_kernel<N, TX, TY, COLLIDE, Pr, true> : fused_step_kernel<N, TX, TY, COLLIDE, Pr>;
+        const int threads = team ? 2 * TX * TY : TX * TY;
+        if (tiles <= sms)
+            return launch_overlapped(kernel, tiles, threads, 0, st, P, pin, pout, (const TA*)ain, (TA*)aout, ex, rows);
+        kernel<<<tiles, threads, 0, st>>>(P, pin, pout, (const TA*)ain, (TA*)aout, ex, rows);
+        return cudaGetLastError();
     }
     return launch_overlapped(fused_step_kernel<N, TX, TY, COLLIDE, Pr>, tiles, TX * TY, 0, st, P, pin, pout, (const TA*)ain,
                              (TA*)aout, ex, rows);
@@ -197,7 +199,9 @@ static cudaError_t launch_batch_step_t(const BatchTable& T, int s, cudaStream_t 
 {
     if constexpr (std::is_same<Pr, PrecFP64>::value) {
         if (fp64_small_tiles(T.total_tiles, T.total_subtiles, T.sms)) {
-            batch_substep_kernel<N, TX, TY, Pr><<<T.total_tiles * BATCH_SUB, BATCH_NT / BATCH_SUB, 0, st>>>(T, s);
+            const bool team = fp64_ring_team(T.total_subtiles, T.sms);
+            const auto kernel = team ? batch_substep_kernel<N, TX, TY, Pr, true> : batch_substep_kernel<N, TX, TY, Pr, false>;
+            kernel<<<T.total_tiles * BATCH_SUB, BATCH_NT / BATCH_SUB * (team ? 2 : 1), 0, st>>>(T, s);
             return cudaGetLastError();
         }
     }

@@ -40,6 +40,14 @@ inline bool fp64_small_tiles(long long tiles, long long subtiles, int sms)
 {
     return (subtiles + sms - 1) / sms * (6 + 1) < (tiles + sms - 1) / sms * (8 * 6 + 3);
 }
+// Whether the 8x4 tiles of an FP64 step take two warps each, one for the cells and one for the ring.
+// A warp alone forms the moments of its cells, then those of the ring's 28 positions, on one
+// scheduler's share of the FP64 unit; a second warp, on another scheduler, halves that stage.  With
+// up to four tiles to an SM (two warps to a scheduler) it was faster at every size tried, N = 2, 3
+// and 4; with more the schedulers are busy anyway, and the second warp's registers cost resident tiles.
+// Measured, us per step, one warp / two: film 16 x 256 23.8 / 20.1; N = 3, 128^2 30.8 / 28.7; N = 4, 112^2
+// 43.9 / 38.4, 128^2 46.1 / 42.0; beyond four tiles N = 3, 224^2 61.5 / 65.6, 300 x 150 59.4 / 65.6.
+inline bool fp64_ring_team(long long tiles, int sms) { return tiles <= 4LL * sms; }
 inline int fp64_tile(int nx, int ny, int sms)
 {
     const long long big = (long long)((nx + 31) / 32) * ((ny + 7) / 8), small = (long long)((nx + 7) / 8) * ((ny + 3) / 4);

@@ -447,14 +447,15 @@ __device__ __forceinline__ void fill_ghosts(const KParams& P, V* fields, int x0,
 // One TX x TY tile (tile column bx, row by) of one time step, run by a block of
 // TX * TY threads; smem holds tile_smem_elems<N, TX, TY, Pr>() elements of shared memory.
 // Every thread of the block must call it (it holds two block barriers); the caller
-// places a block barrier before smem is used again.
-template <int N, int TX, int TY, bool COLLIDE, class Pr, class L>
+// places a block barrier before smem is used again.  RING_TEAM: a block of 2 TX TY threads, whose
+// second half evaluates the ring while the first evaluates the tile's cells (not for COMPACT policies).
+template <int N, int TX, int TY, bool COLLIDE, class Pr, bool RING_TEAM = false, class L>
 __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void* __restrict__ pout_base,
                                             typename Pr::TA* __restrict__ aout, const ExportPtrs& ex, int bx, int by,
                                             typename Pr::R* smem)
 {
     using V = val_t<typename Pr::R>;
-    constexpr int W = TX + 2, H = TY + 2, NT = TX * TY;
+    constexpr int W = TX + 2, H = TY + 2, CELLS = TX * TY, NT = RING_TEAM ? 2 * CELLS : CELLS;
     V* fields = reinterpret_cast<V*>(smem);
     V (*s_phi)[H][W] = reinterpret_cast<V (*)[H][W]>(fields);          // [N][H][W]
     V (*s_rho)[W] = reinterpret_cast<V (*)[W]>(fields + N * H * W);    // [H][W]
@@ -466,7 +467,9 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
     const int tx = tid % TX, ty = tid / TX;
     const int x0 = bx * TX, y0 = by * TY;
     const int x = x0 + tx, y = y0 + ty;
-    const bool owned = x < nx && y < ny;
+    static_assert(!(RING_TEAM && Pr::COMPACT), "the one loop over all positions has no ring of its own");
+    const bool own_team = !RING_TEAM || tid < CELLS;
+    const bool owned = own_team && x < nx && y < ny;
     const bool xper = P.bc[0] == PERIODIC, yper = P.bc[2] == PERIODIC;
     using Cell = typename L::Cell;
 
@@ -533,11 +536,12 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
         if (owned) {
             cell_moments<N, Pr>(P, ld, ld.own(x, y, tx, ty), phi, rhoH, fl);
             share(tx + 1, ty + 1, phi, fl);
-        } else {
+        } else if (own_team) {
             halo_at(tx + 1, ty + 1);
         }
         constexpr int NRING = 2 * W + 2 * TY;
-        for (int k = tid; k < NRING; k += NT) {
+        for (int k = RING_TEAM ? tid - CELLS : tid; k < NRING; k += CELLS) {
+            if (RING_TEAM && own_team) break;
             int lx, ly;
             if (k < W) { lx = k; ly = 0; }
             else if (k < 2 * W) { lx = k - W; ly = H - 1; }
@@ -569,14 +573,14 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
 }
 
 // One TX x TY tile read from global memory (the loader of the one-cell step).
-template <int N, int TX, int TY, bool COLLIDE, class Pr>
+template <int N, int TX, int TY, bool COLLIDE, class Pr, bool RING_TEAM = false>
 __device__ __forceinline__ void step_tile(const KParams& P, const void* __restrict__ pin_base,
                                           void* __restrict__ pout_base, const typename Pr::TA* __restrict__ ain,
                                           typename Pr::TA* __restrict__ aout, const ExportPtrs& ex, int bx, int by,
                                           typename Pr::R* smem)
 {
     const GlobalLoader<Pr> ld{P, pop_view<Pr>(P, pin_base), ain};
-    step_tile_l<N, TX, TY, COLLIDE, Pr>(P, ld, pout_base, aout, ex, bx, by, smem);
+    step_tile_l<N, TX, TY, COLLIDE, Pr, RING_TEAM>(P, ld, pout_base, aout, ex, bx, by, smem);
 }
 
 // Tile (bx, by) of block b of a one-dimensional grid of tx * ty tiles.  The tiles on the
@@ -623,8 +627,8 @@ __device__ __forceinline__ void tile_of_block(int b, int tx, int ty, const TileR
 
 // One launch = one time step of one lattice (or of some of its tile rows, `rows`), one
 // block per tile (a one-dimensional grid, the tiles at the sides first).
-template <int N, int TX, int TY, bool COLLIDE, class Pr>
-__global__ void __launch_bounds__(TX * TY, (LBM_OCC(Pr) + TX * TY - 1) / (TX * TY))
+template <int N, int TX, int TY, bool COLLIDE, class Pr, bool RING_TEAM = false>
+__global__ void __launch_bounds__(TX * TY * (RING_TEAM ? 2 : 1), (LBM_OCC(Pr) + TX * TY - 1) / (TX * TY * (RING_TEAM ? 2 : 1)))
 fused_step_kernel(const KParams P, const void* __restrict__ pin_base, void* __restrict__ pout_base,
                   const typename Pr::TA* __restrict__ ain, typename Pr::TA* __restrict__ aout, ExportPtrs ex,
                   TileRows rows)
@@ -633,7 +637,7 @@ fused_step_kernel(const KParams P, const void* __restrict__ pin_base, void* __re
     int bx, by;
     tile_of_block(blockIdx.x, (P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY, rows, bx, by);
     step_wait_previous();
-    step_tile<N, TX, TY, COLLIDE, Pr>(P, pin_base, pout_base, ain, aout, ex, bx, by, smem);
+    step_tile<N, TX, TY, COLLIDE, Pr, RING_TEAM>(P, pin_base, pout_base, ain, aout, ex, bx, by, smem);
 }
 
 }  // namespace lbm

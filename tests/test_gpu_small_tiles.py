@@ -15,6 +15,7 @@ CASES = {
     "periodic_9x5": lambda: W.perturbed(W.periodic_drop(n=9, R=2.0, ny=5, rho_gas=0.5), seed=2),
     "cap_33x31": lambda: W.sessile_cap(33, 31, 9.0, theta=70.0, ste=0.2),
     "walls_40x40_N3": lambda: _walls(W.lateral_pool(n=40)),
+    "cap_152x150": lambda: W.sessile_cap(152, 150, 40.0, theta=70.0, ste=0.2),   # more than four tiles to an SM
     "walls_65x65_N4": lambda: W.impurity_freeze(n=65, n_disks=2),
 }
 
