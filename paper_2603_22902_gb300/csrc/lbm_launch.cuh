@@ -33,7 +33,7 @@ inline bool tile_dims(int id, int& tx, int& ty)
 // cell's update takes about six times the instructions of a ring position's moments, and a tile
 // of 8 warps has 3 warps of ring positions, a tile of one warp one.  The small tiles cost a tenth
 // more where every SM is full and win where the large ones leave SMs idle or unevenly filled.
-// Measured, us per step, 8x4 against 32x8 (N = 2): 16 x 256 26.1 / 39.8, 128^2 28.6 / 38.0, 192^2
+// Measured, us per step, 8x4 with one warp against 32x8, launches not overlapped (N = 2): 16 x 256 26.1 / 39.8, 128^2 28.6 / 38.0, 192^2
 // 41.1 / 38.6, 256^2 57.4 / 59.5, 384^2 117.5 / 114.5, 448^2 160 / 166, 512^2 201 / 193; the rule takes
 // the faster one at each of these, and for N = 3 and 4.
 inline bool fp64_small_tiles(long long tiles, long long subtiles, int sms)
