@@ -277,10 +277,8 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
     P.d.omega_g = 1.0 / tau_g;
     P.d.kg = 1.0 - 0.5 * P.d.omega_g;
     P.d.omega_g1 = 1.0 - P.d.omega_g;
-    const double gc[5] = {3.0 * (P.d.omega_g + P.d.kg), -3.0 * P.d.kg, P.d.kg, P.d.omega_g, P.d.kg};
-    for (int k = 0; k < 5; ++k) P.d.g_sc[k] = gc[k];
+    const double gc[3] = {3.0 * (P.d.omega_g + P.d.kg), -3.0 * P.d.kg, P.d.kg};
     for (int k = 0; k < 3; ++k) P.d.g_pl[k] = gc[k] / 9.0;
-    P.d.E_ref49 = 4.0 / 9.0 * P.d.E_ref;
     P.ordered = th->T_sol <= 0.0 && th->T_liq >= 0.0 ? 1 : 0;
 
     const size_t pb = plane_bytes(h);

@@ -1,7 +1,7 @@
 // lbm_cell.cuh -- the arithmetic of one lattice update (arXiv 2603.22902, Sections 2 and 3),
 // from the moments of the cell to its post-collision populations and lagged values, written
-// once for every value type (lbm_vals.cuh).  The kernels supply the inputs and take the
-// outputs through an Io object.
+// once for FP64, double words and FP32 (lbm_vals.cuh); 16-bit storage has a form of its own
+// (lbm_cell16.cuh).  The kernels supply the inputs and take the outputs through an Io object.
 //
 // What bounds it: the FP64 policy the number of its FP64 instructions (a warp instruction holds
 // the SM's 2-lane unit for 16 cycles), double words and the FP32-arithmetic policies the number
@@ -14,11 +14,9 @@
 //   * S - 3/2 tr Lambda = -3 u.F, since Lambda = uF + Fu + (S/3) I: S drops out of F_0 and of
 //     the isotropic part of the flow source;
 //   * opposite directions share their even and odd parts in c_i, which carry the weight of the
-//     axis directions (1/9) from the start; SCALED policies hold populations divided by their
-//     weights and need no weights at all.
+//     axis directions (1/9) from the start.
 // Measured at N = 2, 512 x 512 (ncu, one step): FP64 487 -> 365 FP64 instructions per cell and
-// 254 -> 193 us; double words 5600 -> 4740 instructions per cell, 69 -> 62 us; FP16 storage 1440
-// -> 1236 instructions, 20.0 -> 18.7 us.  Against the scheme in long double the FP64 fields
+// 254 -> 193 us; double words 5600 -> 4740 instructions per cell, 69 -> 62 us.  Against the scheme in long double the FP64 fields
 // are 2 to 15 times closer than with one product per weight and direction (the rest direction now
 // takes what the others leave, so that sum_i g_i and sum_i h_i do not drift with the rounding of
 // the weights), double words as close as before.
@@ -52,18 +50,12 @@ __device__ __forceinline__ bool all_equal(V a, float b)
 {
     return a == V(b);
 }
-// x1 where f_l = 1, x0 where f_l = 0, xm elsewhere
-template <class V>
-__device__ __forceinline__ V by_phase(V fl, V x1, V x0, V xm)
-{
-    return fl == V(1.0f) ? x1 : fl == V(0.0f) ? x0 : xm;
-}
 
 // Post-collision populations q_i = (1 - omega) f_i + even_i +- odd_i of the eight moving
 // directions.  ex, ey: even parts of the axis directions; e5, e6: of the diagonals (1, 1) and
-// (-1, 1); odd parts along x and y: ca tx, ca ty.  Plain populations: all parts carry the axis
-// weight 1/9, and the diagonals take a quarter of it.
-template <bool SC, class V, class CA>
+// (-1, 1); odd parts along x and y: ca tx, ca ty.  All parts carry the axis weight 1/9, and the
+// diagonals take a quarter of it.
+template <class V, class CA>
 __device__ __forceinline__ void collide_pairs(V om1, const V (&f)[9], V ex, V ey, V e5, V e6, V tx, V ty, CA ca, V (&q)[9])
 {
     const auto quarter = exact_t<V>(0.25);
@@ -87,58 +79,34 @@ __device__ __forceinline__ void collide_pairs(V om1, const V (&f)[9], V ex, V ey
     q[3] = rfma(om1, f[3], rfma(mx, ca, ex));
     q[2] = rfma(om1, f[2], rfma(ty, ca, ey));
     q[4] = rfma(om1, f[4], rfma(my, ca, ey));
-    if constexpr (SC) {
-        const V o5 = tx + ty, o6 = ty - tx;
-        q[5] = rfma(om1, f[5], rfma(o5, ca, e5));
-        q[7] = rfma(om1, f[7], rfma(-o5, ca, e5));
-        q[6] = rfma(om1, f[6], rfma(o6, ca, e6));
-        q[8] = rfma(om1, f[8], rfma(-o6, ca, e6));
-    } else {
-        const V o5 = (tx + ty) * (ca * quarter), o6 = (ty - tx) * (ca * quarter);
-        q[5] = rfma(om1, f[5], rfma(e5, quarter, o5));
-        q[7] = rfma(om1, f[7], rfma(e5, quarter, -o5));
-        q[6] = rfma(om1, f[6], rfma(e6, quarter, o6));
-        q[8] = rfma(om1, f[8], rfma(e6, quarter, -o6));
-    }
+    const V o5 = (tx + ty) * (ca * quarter), o6 = (ty - tx) * (ca * quarter);
+    q[5] = rfma(om1, f[5], rfma(e5, quarter, o5));
+    q[7] = rfma(om1, f[7], rfma(e5, quarter, -o5));
+    q[6] = rfma(om1, f[6], rfma(e6, quarter, o6));
+    q[8] = rfma(om1, f[8], rfma(e6, quarter, -o6));
 }
 // The same with ca = 1 and one even part e for all directions.
-template <bool SC, class V>
+template <class V>
 __device__ __forceinline__ void collide_pairs(V om1, const V (&f)[9], V e, V ax, V ay, V (&q)[9])
 {
     q[1] = rfma(om1, f[1], e + ax);
     q[3] = rfma(om1, f[3], e - ax);
     q[2] = rfma(om1, f[2], e + ay);
     q[4] = rfma(om1, f[4], e - ay);
-    V o5 = ax + ay, o6 = ay - ax;
-    if constexpr (SC || std::is_same<V, df64>::value) {
-        if constexpr (!SC) {
-            const auto quarter = exact_t<V>(0.25);
-            e = e * quarter;
-            o5 = o5 * quarter;
-            o6 = o6 * quarter;
-        }
+    const auto quarter = exact_t<V>(0.25);
+    const V o5 = (ax + ay) * quarter, o6 = (ay - ax) * quarter;
+    if constexpr (std::is_same<V, df64>::value) {
+        e = e * quarter;
         q[5] = rfma(om1, f[5], e + o5);
         q[7] = rfma(om1, f[7], e - o5);
         q[6] = rfma(om1, f[6], e + o6);
         q[8] = rfma(om1, f[8], e - o6);
     } else {
-        const auto quarter = exact_t<V>(0.25);
-        o5 = o5 * quarter;
-        o6 = o6 * quarter;
         q[5] = rfma(om1, f[5], rfma(e, quarter, o5));
         q[7] = rfma(om1, f[7], rfma(e, quarter, -o5));
         q[6] = rfma(om1, f[6], rfma(e, quarter, o6));
         q[8] = rfma(om1, f[8], rfma(e, quarter, -o6));
     }
-}
-
-// Weight of the rest direction of f relative to the parts of collide_pairs: 4/9 times the scale of
-// the moving populations where they are scaled, 4 where the parts carry 1/9.
-template <bool SC, class V>
-__device__ __forceinline__ constexpr auto rest_weight(double scale)
-{
-    if constexpr (SC) return cst<V>(4.0 / 9.0 * scale);
-    else return exact_t<V>(4);
 }
 
 // sum_p phi_p a_p.
@@ -207,29 +175,23 @@ __device__ __forceinline__ V liquid_fraction(const KParams& P, const V (&phi)[N]
 }
 
 // phi_p and rho H of a cell from its populations and lagged mdot', Q' (Section 3, recovery of
-// phi_p and H).  Plain populations add up; those divided by their weights (SCALED) are weighted
-// per kind of direction.  1 - mdot'/2 divides nothing where mdot' = 0 (away from the front).
-template <int N, bool SCALED, class V, class G, class H>
+// phi_p and H).  1 - mdot'/2 divides nothing where mdot' = 0 (away from the front).
+template <int N, class V, class G, class H>
 __device__ __forceinline__ void moments(const KParams& P, V mdm, V Qm, G&& g, H&& h, V (&phi)[N], V& rhoH)
 {
     using K = exact_t<V>;
-    auto sum = [](auto&& q, auto scale) {
+    auto sum = [](auto&& q) {
         const V a = (q(1) + q(3)) + (q(2) + q(4)), d = (q(5) + q(7)) + (q(6) + q(8));
-        if constexpr (SCALED) {
-            // rest + (a / 9 + d / 36) scale
-            return rfma(rfma(d, 0.25f, a), cst<V>(1.0 / 9.0) * scale, q(0));
-        } else {
-            return q(0) + (a + d);
-        }
+        return q(0) + (a + d);
     };
 #pragma unroll
-    for (int p = 0; p < N; ++p) phi[p] = sum([&](int i) { return g(p, i); }, 1.0f);
+    for (int p = 0; p < N; ++p) phi[p] = sum([&](int i) { return g(p, i); });
     if (any_nonzero(mdm)) {
         const V iden = rinv(rfma(mdm, K(-0.5), V(K(1))));
 #pragma unroll
         for (int p = 0; p < N; ++p) phi[p] = phi[p] * iden;
     }
-    rhoH = rfma(Qm, K(0.5), sum([&](int i) { return h(i); }, coef<const_t<V>>(P).E_ref));
+    rhoH = rfma(Qm, K(0.5), sum([&](int i) { return h(i); }));
 }
 
 // The mixture of eq. 2 in one cell.
@@ -294,10 +256,8 @@ __device__ __forceinline__ Mixture<V> mixture_of(const KParams& P, const V (&phi
         m.cp = rfma(fs, phi_sum<N>(phi, C.cp_s), fl * phi_sum<N>(phi, C.cp_l));
         m.psi = fs * phi_sum<N>(phi, C.drho);
         m.chi = fs * phi_sum<N>(phi, C.pcm);
-        // T_sol + f_l (T_liq - T_sol) in the mushy band (in f2 some lanes may be pure)
-        const V liquid = liquid_sensible<N>(phi, rhoH, C.rhoL);
-        m.Zn = by_phase(fl, liquid, rhoH, zero);
-        m.T0 = by_phase(fl, zero, zero, rfma(fl, C.T_liq - C.T_sol, V(C.T_sol)));
+        m.Zn = zero;
+        m.T0 = rfma(fl, C.T_liq - C.T_sol, V(C.T_sol));
     }
     return m;
 }
@@ -335,20 +295,19 @@ __device__ __forceinline__ V normal_weight(V s, V G2, V ref, V a)
     return r;
 }
 
-// The update of one cell (two for f2), stages C to G.  phi, rhoH, fl: its moments and liquid
+// The update of one cell, stages C to G.  phi, rhoH, fl: its moments and liquid
 // fraction.  Io supplies
 //   stencil(fi, gx, gy, lap): 12 grad of field fi (phi_p: fi = p, rho: N, psi: N + 1), and
-//     6 lap for fi < N;   f(i), g(p, i), h(i): its populations (divided by their weights and
-//     scales for SCALED policies, except i = 0);   lag(a): lagged plane a (see aux_psi ...);
+//     6 lap for fi < N;   f(i), g(p, i), h(i): its populations;   lag(a): lagged plane a (see
+//     aux_psi ...);
 // and takes
-//   push<KIND>(s, q): the post-collision populations of species s (in the same form);
+//   push<KIND>(s, q): the post-collision populations of species s;
 //   dirichlet(...): the boundary row's incoming enthalpy populations;
 //   put_lag(a, v): the lagged values;   put_fields(...): the macroscopic fields (!COLLIDE).
 template <int N, bool COLLIDE, class Pr, class V, class Io>
 __device__ __forceinline__ void cell_update(const KParams& P, Io& io, const V (&phi)[N], V rhoH, V fl)
 {
     using K = exact_t<V>;
-    constexpr bool SC = Pr::QUANT;
     const auto& C = coef<const_t<V>>(P);
     const Mixture<V> m = mixture_of<N>(P, phi, rhoH, fl);
     const V rho = m.rho;
@@ -410,17 +369,9 @@ __device__ __forceinline__ void cell_update(const KParams& P, Io& io, const V (&
 #pragma unroll
     for (int i = 0; i < 9; ++i) f[i] = io.f(i);
     const V fa = f[5] - f[7], fb = f[8] - f[6];
-    V jx, jy, sum_f;
-    if constexpr (SC) {
-        const float wa = F_SCALE / 9.0f;
-        jx = rfma(fa + fb, 0.25f, f[1] - f[3]) * wa;
-        jy = rfma(fa - fb, 0.25f, f[2] - f[4]) * wa;
-        sum_f = rfma((f[5] + f[6]) + (f[7] + f[8]), 0.25f, (f[1] + f[2]) + (f[3] + f[4])) * wa;
-    } else {
-        jx = (f[1] - f[3]) + (fa + fb);
-        jy = (f[2] - f[4]) + (fa - fb);
-        sum_f = ((f[1] + f[2]) + (f[3] + f[4])) + ((f[5] + f[6]) + (f[7] + f[8]));
-    }
+    const V jx = (f[1] - f[3]) + (fa + fb);
+    const V jy = (f[2] - f[4]) + (fa - fb);
+    const V sum_f = ((f[1] + f[2]) + (f[3] + f[4])) + ((f[5] + f[6]) + (f[7] + f[8]));
     // 1 / rho, omega_f = 1 / tau_f = rho / A, omega_h = 1 / tau_h = 1 / B and T = Zn / (rho c_p) + T0;
     // tau_f = A / rho, A = 3 mu + rho / 2 (tau_f = mu / (rho c_s^2) + 1/2), and
     // tau_h = B = lambda / (rho_ref c_p,ref c_s^2) + 1/2
@@ -464,60 +415,45 @@ __device__ __forceinline__ void cell_update(const KParams& P, Io& io, const V (&
     }
 
     // ---- stage F: flow collision -------------------------------------------
-    // even and odd parts of the equilibrium and source terms over w_i, times 1/9 for plain
-    // populations (and over F_SCALE for scaled ones)
+    // even and odd parts of the equilibrium and source terms over w_i, times 1/9
     {
-        V oms = om, ks = rfma(om, K(-0.5), V(K(1)));
-        const V om1 = V(K(1)) - om;
-        V ex = ux, ey = uy;
-        if constexpr (SC) {
-            oms = om * (1.0f / F_SCALE);
-            ks = ks * (1.0f / F_SCALE);
-            ex = ux * 9.0f;
-            ey = uy * 9.0f;
-        }
-        const V rom = oms * rho, krho = ks * rho;
+        const V ks = rfma(om, K(-0.5), V(K(1))), om1 = V(K(1)) - om;
+        const V rom = om * rho, krho = ks * rho;
         const V hrom = rom * K(0.5), kFx = ks * Fx, kFy = ks * Fy;
         const V X = rfma(hrom, ux, kFx), Y = rfma(hrom, uy, kFy);
-        const V axy = rfma(ex, Y, ey * X);
+        const V axy = rfma(ux, Y, uy * X);
         const V kS = ks * S;
-        const auto cs = cst<V>(SC ? 1.5 : 1.0 / 6.0);
-        const V omp = oms * p;
-        const V iso = rfma(ex, X, ey * Y) * cst<V>(-1.0 / 3.0);
-        const V a0 = rfma(omp, cst<V>(SC ? 3.0 : 1.0 / 3.0), iso);
-        const V x0 = rfma(omp, cst<V>(SC ? -3.75 : -3.75 / 9.0), iso);
+        const auto sixth = cst<V>(1.0 / 6.0), third = cst<V>(1.0 / 3.0);
+        const V omp = om * p;
+        const V iso = rfma(ux, X, uy * Y) * cst<V>(-1.0 / 3.0);
+        const V a0 = rfma(omp, third, iso);
+        const V x0 = rfma(omp, cst<V>(-3.75 / 9.0), iso);
         const V tx = rfma(krho, fpx, rfma(rom, ux, kFx)), ty = rfma(krho, fpy, rfma(rom, uy, kFy));
-        const V as = rfma(kS, cs, a0), bx = rfma(ex, X, as), by = rfma(ey, Y, as), bd = rfma(kS, cs, rfma(ey, Y, bx));
+        const V as = rfma(kS, sixth, a0), bx = rfma(ux, X, as), by = rfma(uy, Y, as), bd = rfma(kS, sixth, rfma(uy, Y, bx));
         V q[9];
-        q[0] = rfma(x0, rest_weight<SC, V>(F_SCALE), om1 * f[0]);
-        collide_pairs<SC>(om1, f, bx, by, bd + axy, bd - axy, tx, ty, cst<V>(SC ? 3.0 : 1.0 / 3.0), q);
+        q[0] = rfma(x0, K(4), om1 * f[0]);
+        collide_pairs(om1, f, bx, by, bd + axy, bd - axy, tx, ty, third, q);
         io.template push<KIND_F>(0, q);
     }
 
     // ---- stage F: phase-field collisions -------------------------------------
     {
-        const auto& cg = SC ? C.g_sc : C.g_pl;
-        const V gm = rfma(mdot, C.g_sc[4], V(C.g_sc[3]));
+        const V gm = rfma(mdot, C.kg, V(C.omega_g));
 #pragma unroll(Pr::COMPACT ? 1 : N)
         for (int pp = 0; pp < N; ++pp) {
             V gq[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i) gq[i] = io.g(pp, i);
             const V pu = phi[pp] * ux, pv = phi[pp] * uy;
-            const V bx = rfma(pu, cg[0], rfma(io.lag(aux_phiux(pp)), cg[1], Rx[pp] * cg[2]));
-            const V by = rfma(pv, cg[0], rfma(io.lag(aux_phiuy(N, pp)), cg[1], Ry[pp] * cg[2]));
+            const V bx = rfma(pu, C.g_pl[0], rfma(io.lag(aux_phiux(pp)), C.g_pl[1], Rx[pp] * C.g_pl[2]));
+            const V by = rfma(pv, C.g_pl[0], rfma(io.lag(aux_phiuy(N, pp)), C.g_pl[1], Ry[pp] * C.g_pl[2]));
             const V og1 = V(C.omega_g1);
-            V b0 = phi[pp] * gm, q[9];
-            if constexpr (SC) {
-                q[0] = rfma(b0, rest_weight<SC, V>(1.0), gq[0] * C.omega_g1);
-            } else {
-                // the rest direction takes what the others leave of phi_p (omega_g + k_g mdot), so
-                // that the rounding of 1/9 does not change sum_i g_i, step after step
-                const V all = b0;
-                b0 = b0 * cst<V>(1.0 / 9.0);
-                q[0] = rfma(b0, K(-5), rfma(gq[0], C.omega_g1, all));
-            }
-            collide_pairs<SC>(og1, gq, b0, bx, by, q);
+            // the rest direction takes what the others leave of phi_p (omega_g + k_g mdot), so
+            // that the rounding of 1/9 does not change sum_i g_i, step after step
+            const V all = phi[pp] * gm, b0 = all * cst<V>(1.0 / 9.0);
+            V q[9];
+            q[0] = rfma(b0, K(-5), rfma(gq[0], C.omega_g1, all));
+            collide_pairs(og1, gq, b0, bx, by, q);
             io.template push<KIND_G>(1 + pp, q);
             io.put_lag(aux_phiux(pp), pu);
             io.put_lag(aux_phiuy(N, pp), pv);
@@ -529,35 +465,23 @@ __device__ __forceinline__ void cell_update(const KParams& P, Io& io, const V (&
         V h[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) h[i] = io.h(i);
-        // Z = rho c_p T, E = rho_ref c_p,ref T; scaled populations are over rho_ref c_p,ref as well
+        // Z = rho c_p T, E = rho_ref c_p,ref T
         const V Z = rfma(rc, m.T0, m.Zn), E = T * C.E_ref;
         const V kh = rfma(oh, K(-0.5), V(K(1))), oh1 = V(K(1)) - oh;
-        const V Zm = Z * mdot;
-        V Zs = Z, src, base;
-        if constexpr (SC) {
-            Zs = Z * C.inv_E_ref;
-            src = kh * (Zs * mdot);
-            base = rfma(oh, T, src);
-        } else {
-            src = kh * Zm;
-            base = rfma(oh, E, src) * cst<V>(1.0 / 9.0);
-        }
-        const V ohZ = oh * Zs, vx = ohZ * ux, vy = ohZ * uy;
+        const V Zm = Z * mdot, src = kh * Zm;
+        const V base = rfma(oh, E, src) * cst<V>(1.0 / 9.0);
+        const V ohZ = oh * Z, vx = ohZ * ux, vy = ohZ * uy;
         const V vxx = vx * ux, vyy = vy * uy, vs = vxx + vyy;
-        const V c0 = rfma(vs, cst<V>(SC ? -1.5 : -1.0 / 6.0), base);
-        const K half = K(SC ? 4.5 : 0.5);
-        const V bx = rfma(vxx, half, c0), by = rfma(vyy, half, c0), bd = rfma(vs, half, c0);
-        V wy = uy;
-        if constexpr (SC) wy = uy * 9.0f;
+        const V c0 = rfma(vs, cst<V>(-1.0 / 6.0), base);
+        const V bx = rfma(vxx, K(0.5), c0), by = rfma(vyy, K(0.5), c0), bd = rfma(vs, K(0.5), c0);
         V q[9];
-        if constexpr (SC) q[0] = rfma(oh, rhoH - E, rfma(c0, C.E_ref49, oh1 * h[0]));
         // the rest direction takes what the others leave of omega_h rho H + k_h Z mdot
-        else q[0] = rfma(c0, K(-5), rfma(vs, K(-1.5), rfma(oh1, h[0], rfma(oh, rhoH, src))));
-        collide_pairs<SC>(oh1, h, bx, by, rfma(vx, wy, bd), rfma(-vx, wy, bd), vx, vy, cst<V>(SC ? 3.0 : 1.0 / 3.0), q);
+        q[0] = rfma(c0, K(-5), rfma(vs, K(-1.5), rfma(oh1, h[0], rfma(oh, rhoH, src))));
+        collide_pairs(oh1, h, bx, by, rfma(vx, uy, bd), rfma(-vx, uy, bd), vx, vy, cst<V>(1.0 / 3.0), q);
         // outflow rows are copied inside push; Dirichlet rows get their incoming populations
         // from the ghost rule
         io.template push<KIND_H>(N + 1, q);
-        io.dirichlet(h, oh1, Zs, SC ? T : E, T, ux, uy, uu);
+        io.dirichlet(h, oh1, Z, E, T, ux, uy, uu);
         io.put_lag(aux_mdot(), mdot);
         io.put_lag(aux_Q(), Zm);
         io.put_lag(aux_psi(), m.psi);

@@ -54,10 +54,7 @@ struct Coef {
     T us[2], accel[2];
     T omega_g, kg;                // 1 / tau_g and 1 - 1/(2 tau_g), tau_g = M / c_s^2 + 1/2
     T omega_g1;                   // 1 - 1 / tau_g
-    // phase-field collision: 3 (omega_g + k_g), -3 k_g, k_g over 9 for plain populations (g_pl);
-    // as they are for populations divided by their weights, with omega_g, k_g (g_sc)
-    T g_pl[3], g_sc[5];
-    T E_ref49;                    // 4/9 rho_ref c_p,ref
+    T g_pl[3];                    // phase-field collision: 3 (omega_g + k_g), -3 k_g, k_g over 9
     T Tw[4];                      // Dirichlet wall temperature
     T rhoL[MAXN];                 // rho_l^p L_p (the FP64 map reads KParams::rhoL)
     T T_sol, T_liq;               // (the FP64 map reads KParams::T_sol, T_liq)

@@ -69,7 +69,7 @@ struct StageLayout {
 template <int N, class Pr>
 struct StagedLoader {
     using R = typename Pr::R;
-    using V = val_t<R>;
+    using V = step_val<Pr>;
     using TR = typename Pr::TR;
     using TM = typename Pr::TM;
     using TA = typename Pr::TA;
@@ -92,19 +92,25 @@ struct StagedLoader {
         return !(bx || by);
     }
     __device__ __forceinline__ Cell own(int, int, int tx, int ty) const { return (ty + 1) * 64 + tx + 1; }
+    template <int KIND>
     __device__ __forceinline__ V pop(int s, int i, Cell c, int) const
     {
         const int lx = c & 63, ly = c >> 6;
         if (s == 0) {  // the flow populations: own cells only
             const int o = (ly - 1) * STAGE_TX + (lx - 1);
-            if (i == 0) return stored<Pr>(reinterpret_cast<const TR*>(st + Lay::OC)[o]);
-            return stored<Pr>(reinterpret_cast<const TM*>(st + Lay::OA)[(i - 1) * STAGE_TY * STAGE_TX + o]);
+            if (i == 0) return (R) reinterpret_cast<const TR*>(st + Lay::OC)[o];
+            return dequant<Pr, KIND>(P, reinterpret_cast<const TM*>(st + Lay::OA)[(i - 1) * STAGE_TY * STAGE_TX + o], i);
         }
-        if (i == 0) return stored<Pr>(reinterpret_cast<const TR*>(st + Lay::OD)[((s - 1) * Lay::H + ly) * Lay::WR + lx - 1 + Lay::PR]);
+        if (i == 0) return (R) reinterpret_cast<const TR*>(st + Lay::OD)[((s - 1) * Lay::H + ly) * Lay::WR + lx - 1 + Lay::PR];
         const int plane = (s - 1) * 8 + i - 1;
-        return stored<Pr>(reinterpret_cast<const TM*>(st + Lay::OB)[(plane * Lay::H + ly) * Lay::WM + lx - 1 + Lay::PM]);
+        return dequant<Pr, KIND>(P, reinterpret_cast<const TM*>(st + Lay::OB)[(plane * Lay::H + ly) * Lay::WM + lx - 1 + Lay::PM],
+                                 i);
     }
-    __device__ __forceinline__ V pop_late(int s, int i, Cell c, int site) const { return pop(s, i, c, site); }
+    template <int KIND>
+    __device__ __forceinline__ V pop_late(int s, int i, Cell c, int site) const
+    {
+        return pop<KIND>(s, i, c, site);
+    }
     __device__ __forceinline__ V aux(int a, Cell c, int) const
     {
         const int lx = c & 63, ly = c >> 6;

@@ -17,7 +17,7 @@
 //      the cells that are clearly liquid or solid (liquid_fraction, lbm_cell.cuh);
 //   2. ghost values beyond walls/outflows are filled (zero gradient; wetting for phi_p),
 //      skipped by tiles that have none;
-//   3. the rest of the cell's update (cell_update, lbm_cell.cuh): stencils from shared
+//   3. the rest of the cell's update (lbm_cell.cuh, for 16-bit storage lbm_cell16.cuh): stencils from shared
 //      memory, interface terms, flow macroscopics and the three BGK collisions;
 //   4. post-collision populations are pushed to the neighbours' slots of set B with
 //      the boundary rules (bounce-back, outflow copy, non-equilibrium extrapolation
@@ -28,6 +28,7 @@
 #pragma once
 
 #include "lbm_cell.cuh"
+#include "lbm_cell16.cuh"
 #include "lbm_device.cuh"
 #include "lbm_prec.cuh"
 
@@ -83,38 +84,52 @@ __device__ __forceinline__ typename Pr::R ld_pop(const KParams& P, const PopView
     return dequant<Pr, KIND>(P, q, i);
 }
 
-// A stored value as the step's arithmetic takes it: 16-bit moving populations stay divided by
-// their weight and scale (see st_val).
-template <class Pr, class T>
-__device__ __forceinline__ val_t<typename Pr::R> stored(T q)
-{
-    if constexpr (Pr::QUANT && !std::is_same<T, float>::value) return f1(to_f(q));
-    else return val_t<typename Pr::R>((typename Pr::R)q);
-}
-
-// Load population i of species s at cell c in its stored form.
+// The value type of a policy's step: 16-bit storage computes in float (lbm_cell16.cuh).
 template <class Pr>
-__device__ __forceinline__ val_t<typename Pr::R> ld_val(const KParams& P, const PopView<Pr>& v, int s, int i, unsigned c, int site)
+using step_val = typename std::conditional<Pr::QUANT, float, val_t<typename Pr::R>>::type;
+
+// Population i of species s at cell c as the step's arithmetic takes it.
+template <class Pr, int KIND>
+__device__ __forceinline__ step_val<Pr> ld_val(const KParams& P, const PopView<Pr>& v, int s, int i, unsigned c, int site)
 {
-    if (i == 0) return stored<Pr>(ld_plane<Pr::COH>(P, v.rest, s, c, P.rest_elems, site));
-    return stored<Pr>(ld_plane<Pr::COH>(P, v.move, s * 8 + i - 1, c, P.move_elems, site));
+    using R = typename Pr::R;
+    if (i == 0) return step_val<Pr>((R)ld_plane<Pr::COH>(P, v.rest, s, c, P.rest_elems, site));
+    return step_val<Pr>(dequant<Pr, KIND>(P, ld_plane<Pr::COH>(P, v.move, s * 8 + i - 1, c, P.move_elems, site), i));
 }
 
 // The same load for a second read of a population in one step: through the cached
 // (L1) path instead of the read-only one, so that the compiler does not merge it with
 // the first read and keep the value in a register meanwhile.
-template <class Pr>
-__device__ __forceinline__ val_t<typename Pr::R> ld_val_late(const KParams& P, const PopView<Pr>& v, int s, int i, unsigned c, int site)
+template <class Pr, int KIND>
+__device__ __forceinline__ step_val<Pr> ld_val_late(const KParams& P, const PopView<Pr>& v, int s, int i, unsigned c, int site)
 {
+    using R = typename Pr::R;
 #ifdef LBM_CHECK_BOUNDS
     const long long idx = i == 0 ? (long long)s * P.S + c : (long long)(s * 8 + i - 1) * P.S + c;
     if (!lbm_in_bounds(P.dbg, idx, i == 0 ? P.rest_elems : P.move_elems, site))
-        return val_t<typename Pr::R>((typename Pr::R)0.0f);
+        return step_val<Pr>((R)0.0f);
 #else
     (void)site;
 #endif
-    if (i == 0) return stored<Pr>(lbm_ld_l1<Pr::COH>(plane_elem(v.rest, P, s, c)));
-    return stored<Pr>(lbm_ld_l1<Pr::COH>(plane_elem(v.move, P, s * 8 + i - 1, c)));
+    if (i == 0) return step_val<Pr>((R)lbm_ld_l1<Pr::COH>(plane_elem(v.rest, P, s, c)));
+    return step_val<Pr>(dequant<Pr, KIND>(P, lbm_ld_l1<Pr::COH>(plane_elem(v.move, P, s * 8 + i - 1, c)), i));
+}
+
+// The plain value val of a moving population (direction i >= 1) in its stored form.
+template <class Pr, int KIND>
+__device__ __forceinline__ typename Pr::TM quant(const KParams& P, typename Pr::R val, int i)
+{
+    using TM = typename Pr::TM;
+    if constexpr (!Pr::QUANT) {
+        return (TM)val;
+    } else {
+        const float w = (float)wgt(i);
+        float q;
+        if (KIND == KIND_F) q = (float)val * (1.0f / (w * F_SCALE));
+        else if (KIND == KIND_G) q = (float)val * (1.0f / w);
+        else q = (float)val * (1.0f / w) * P.f.inv_E_ref;
+        return from_f<TM>(q);
+    }
 }
 
 // Store the plain value val of population i of species s at cell c (quantised from R).
@@ -122,37 +137,20 @@ template <class Pr, int KIND>
 __device__ __forceinline__ void st_pop(const KParams& P, const PopView<Pr>& v, int s, int i, long long c,
                                        typename Pr::R val, int site)
 {
-    using TM = typename Pr::TM;
-    if (i == 0) {
-        LBM_ST(P, v.rest, (long long)s * P.S + c, P.rest_elems, site, (typename Pr::TR)val);
-        return;
-    }
-    const long long idx = (long long)(s * 8 + i - 1) * P.S + c;
-    if constexpr (!Pr::QUANT) {
-        LBM_ST(P, v.move, idx, P.move_elems, site, (TM)val);
-    } else {
-        const float w = (float)wgt(i);
-        float q;
-        if (KIND == KIND_F) q = (float)val * (1.0f / (w * F_SCALE));
-        else if (KIND == KIND_G) q = (float)val * (1.0f / w);
-        else q = (float)val * (1.0f / w) * P.f.inv_E_ref;
-        LBM_ST(P, v.move, idx, P.move_elems, site, from_f<TM>(q));
-    }
+    if (i == 0) LBM_ST(P, v.rest, (long long)s * P.S + c, P.rest_elems, site, (typename Pr::TR)val);
+    else LBM_ST(P, v.move, (long long)(s * 8 + i - 1) * P.S + c, P.move_elems, site, (quant<Pr, KIND>(P, val, i)));
 }
 
-// Store population i of species s at cell c + shift from its stored form: the plain value, or for
-// the 16-bit policies f_i / (w_i F_SCALE), g_i / w_i, h_i / (w_i rho_ref c_p,ref) of a moving direction
-// and the plain value of the rest direction.  shift is the same for all threads.
-template <class Pr>
+// The same at cell c + shift, from the step's value type; shift is the same for all threads.
+template <class Pr, int KIND>
 __device__ __forceinline__ void st_val(const KParams& P, const PopView<Pr>& v, int s, int i, int shift, unsigned c,
-                                       val_t<typename Pr::R> val, int site)
+                                       step_val<Pr> val, int site)
 {
     using R = typename Pr::R;
     using TR = typename Pr::TR;
     using TM = typename Pr::TM;
     if (i == 0) st_plane<TR>(P, v.rest, s, shift, c, P.rest_elems, site, (TR)(R)val);
-    else if constexpr (!Pr::QUANT) st_plane<TM>(P, v.move, s * 8 + i - 1, shift, c, P.move_elems, site, (TM)(R)val);
-    else st_plane<TM>(P, v.move, s * 8 + i - 1, shift, c, P.move_elems, site, from_f<TM>((R)val));
+    else st_plane<TM>(P, v.move, s * 8 + i - 1, shift, c, P.move_elems, site, quant<Pr, KIND>(P, (R)val, i));
 }
 
 // Where a step reads its inputs.  A loader addresses a cell of the tile-with-ring by a
@@ -163,17 +161,22 @@ __device__ __forceinline__ void st_val(const KParams& P, const PopView<Pr>& v, i
 //     tensor-memory accelerator (lbm_staged.cuh); cells by their position in the tile.
 template <class Pr>
 struct GlobalLoader {
-    using V = val_t<typename Pr::R>;
+    using V = step_val<Pr>;
     using Cell = unsigned;
     static constexpr bool GLOBAL = true;   // step_tile_l locates the cells itself
     const KParams& P;
     PopView<Pr> pin;
     const typename Pr::TA* __restrict__ ain;
     __device__ __forceinline__ Cell own(int x, int y, int, int) const { return (unsigned)y * (unsigned)P.nx + (unsigned)x; }
-    __device__ __forceinline__ V pop(int s, int i, Cell c, int site) const { return ld_val<Pr>(P, pin, s, i, c, site); }
+    template <int KIND>
+    __device__ __forceinline__ V pop(int s, int i, Cell c, int site) const
+    {
+        return ld_val<Pr, KIND>(P, pin, s, i, c, site);
+    }
+    template <int KIND>
     __device__ __forceinline__ V pop_late(int s, int i, Cell c, int site) const
     {
-        return ld_val_late<Pr>(P, pin, s, i, c, site);
+        return ld_val_late<Pr, KIND>(P, pin, s, i, c, site);
     }
     __device__ __forceinline__ V aux(int a, Cell c, int site) const
     {
@@ -185,8 +188,9 @@ struct GlobalLoader {
 template <int N, class Pr, class L, class V>
 __device__ __forceinline__ void cell_moments(const KParams& P, const L& ld, typename L::Cell c, V (&phi)[N], V& rhoH, V& fl)
 {
-    moments<N, Pr::QUANT>(P, ld.aux(aux_mdot(), c, 1), ld.aux(aux_Q(), c, 2), [&](int p, int i) { return ld.pop(1 + p, i, c, 3); },
-                          [&](int i) { return ld.pop(N + 1, i, c, 4); }, phi, rhoH);
+    moments<N>(P, ld.aux(aux_mdot(), c, 1), ld.aux(aux_Q(), c, 2),
+               [&](int p, int i) { return ld.template pop<KIND_G>(1 + p, i, c, 3); },
+               [&](int i) { return ld.template pop<KIND_H>(N + 1, i, c, 4); }, phi, rhoH);
     fl = liquid_fraction<N>(P, phi, rhoH);
 }
 
@@ -209,7 +213,7 @@ __device__ __forceinline__ void halo_moments(const KParams& P, const PopView<Pr>
 // the enthalpy populations at a Dirichlet wall (their incoming slots are filled by the
 // ghost rule); through an outflow side it is dropped.
 template <int J, int KIND, class Pr>
-__device__ __forceinline__ void push(const KParams& P, const PopView<Pr>& out, int s, int x, int y, val_t<typename Pr::R> q)
+__device__ __forceinline__ void push(const KParams& P, const PopView<Pr>& out, int s, int x, int y, step_val<Pr> q)
 {
     int tx = x + cx(J), ty = y + cy(J);
     bool xo = false, yo = false;
@@ -223,13 +227,13 @@ __device__ __forceinline__ void push(const KParams& P, const PopView<Pr>& out, i
     }
     const unsigned own = (unsigned)y * (unsigned)P.nx + (unsigned)x;
     if (!xo && !yo) {
-        st_val<Pr>(P, out, s, J, 0, (unsigned)ty * (unsigned)P.nx + (unsigned)tx, q, 10);
+        st_val<Pr, KIND>(P, out, s, J, 0, (unsigned)ty * (unsigned)P.nx + (unsigned)tx, q, 10);
     } else if (xo) {
-        st_val<Pr>(P, out, s, opp(J), 0, own, q, 11);
+        st_val<Pr, KIND>(P, out, s, opp(J), 0, own, q, 11);
     } else {
         const int side = ty < 0 ? 2 : 3;
         if (P.bc[side] == WALL && !(KIND == KIND_H && P.tbc[side] == DIRICHLET))
-            st_val<Pr>(P, out, s, opp(J), 0, own, q, 12);
+            st_val<Pr, KIND>(P, out, s, opp(J), 0, own, q, 12);
     }
 }
 
@@ -237,27 +241,27 @@ __device__ __forceinline__ void push(const KParams& P, const PopView<Pr>& out, i
 // same row; skipped when that node is beyond an x wall.
 template <int J, int KIND, class Pr>
 __device__ __forceinline__ void push_row(const KParams& P, const PopView<Pr>& out, int s, int x, int y,
-                                         val_t<typename Pr::R> v)
+                                         step_val<Pr> v)
 {
     int tx = x + cx(J);
     if (cx(J) != 0 && (unsigned)tx >= (unsigned)P.nx) {
         if (P.bc[0] != PERIODIC) return;
         tx = tx < 0 ? tx + P.nx : tx - P.nx;
     }
-    st_val<Pr>(P, out, s, J, 0, (unsigned)y * (unsigned)P.nx + (unsigned)tx, v, 13);
+    st_val<Pr, KIND>(P, out, s, J, 0, (unsigned)y * (unsigned)P.nx + (unsigned)tx, v, 13);
 }
 
 // push_row for a direction j known at run time, whose x component is dx.
 template <int KIND, class Pr>
 __device__ __forceinline__ void push_row_at(const KParams& P, const PopView<Pr>& out, int s, int j, int dx, int x,
-                                            int y, val_t<typename Pr::R> v)
+                                            int y, step_val<Pr> v)
 {
     int tx = x + dx;
     if (dx != 0 && (unsigned)tx >= (unsigned)P.nx) {
         if (P.bc[0] != PERIODIC) return;
         tx = tx < 0 ? tx + P.nx : tx - P.nx;
     }
-    st_val<Pr>(P, out, s, j, 0, (unsigned)y * (unsigned)P.nx + (unsigned)tx, v, 13);
+    st_val<Pr, KIND>(P, out, s, j, 0, (unsigned)y * (unsigned)P.nx + (unsigned)tx, v, 13);
 }
 
 // All nine pushes of one species, plus the outflow copies of the boundary rows.  Two paths,
@@ -268,15 +272,15 @@ __device__ __forceinline__ void push_row_at(const KParams& P, const PopView<Pr>&
 //   otherwise the checks of push() for every population.
 template <int KIND, class Pr>
 __device__ __forceinline__ void push_species(const KParams& P, const PopView<Pr>& out, int s, int x, int y,
-                                             bool inside, const val_t<typename Pr::R> (&q)[9])
+                                             bool inside, const step_val<Pr> (&q)[9])
 {
     if (inside) {
         const unsigned nx = (unsigned)P.nx, c = (unsigned)y * nx + (unsigned)x;
         const unsigned cm = x == 0 ? c + (nx - 1) : c - 1, cp = x == P.nx - 1 ? c - (nx - 1) : c + 1;
-        st_val<Pr>(P, out, s, 0, 0, c, q[0], 10);
+        st_val<Pr, KIND>(P, out, s, 0, 0, c, q[0], 10);
 #pragma unroll
         for (int j = 1; j < 9; ++j)
-            st_val<Pr>(P, out, s, j, cy(j) * P.nx, cx(j) < 0 ? cm : (cx(j) > 0 ? cp : c), q[j], 10);
+            st_val<Pr, KIND>(P, out, s, j, cy(j) * P.nx, cx(j) < 0 ? cm : (cx(j) > 0 ? cp : c), q[j], 10);
         return;
     }
     push<0, KIND, Pr>(P, out, s, x, y, q[0]);
@@ -315,12 +319,12 @@ __host__ __device__ constexpr int tile_smem_elems()
     return (N + 2) * (TX + 2) * (TY + 2) + (Pr::COMPACT ? 2 * TX * TY : 0);
 }
 
-// What cell_update (lbm_cell.cuh) reads and writes of the cell (x, y) of a tile: its stencil
+// What cell_update and cell_update16 read and write of the cell (x, y) of a tile: its stencil
 // windows from shared memory (fields of H x W values, the cell at (lx, ly)), its populations and
 // lagged values through the loader, its outputs to set B.
 template <int N, int H, int W, class Pr, class L>
 struct CellIo {
-    using V = val_t<typename Pr::R>;
+    using V = step_val<Pr>;
     using TA = typename Pr::TA;
     const KParams& P;
     const L& ld;
@@ -332,17 +336,24 @@ struct CellIo {
     bool inside;                   // push_species
     unsigned c;
     typename L::Cell oc;
-    __device__ __forceinline__ void stencil(int fi, V& gx, V& gy, V& lap) const
+    // the nine values of field fi around the cell
+    __device__ __forceinline__ void window(int fi, V& c0, V& e, V& w, V& n, V& s, V& ne, V& nw, V& se, V& sw) const
     {
         const V (*a)[W] = reinterpret_cast<const V (*)[W]>(fields + fi * H * W);
-        const V e = a[ly][lx + 1], w = a[ly][lx - 1], n = a[ly + 1][lx], s = a[ly - 1][lx];
-        const V ne = a[ly + 1][lx + 1], nw = a[ly + 1][lx - 1], se = a[ly - 1][lx + 1], sw = a[ly - 1][lx - 1];
-        grad12(e, w, n, s, ne, nw, se, sw, gx, gy);
-        if (fi < N) lap = lap6(a[ly][lx], e, w, n, s, ne, nw, se, sw);
+        e = a[ly][lx + 1], w = a[ly][lx - 1], n = a[ly + 1][lx], s = a[ly - 1][lx];
+        ne = a[ly + 1][lx + 1], nw = a[ly + 1][lx - 1], se = a[ly - 1][lx + 1], sw = a[ly - 1][lx - 1];
+        if (fi < N) c0 = a[ly][lx];
     }
-    __device__ __forceinline__ V f(int i) const { return ld.pop_late(0, i, oc, 5); }
-    __device__ __forceinline__ V g(int p, int i) const { return ld.pop_late(1 + p, i, oc, 6); }
-    __device__ __forceinline__ V h(int i) const { return ld.pop_late(N + 1, i, oc, 7); }
+    __device__ __forceinline__ void stencil(int fi, V& gx, V& gy, V& lap) const
+    {
+        V c0, e, w, n, s, ne, nw, se, sw;
+        window(fi, c0, e, w, n, s, ne, nw, se, sw);
+        grad12(e, w, n, s, ne, nw, se, sw, gx, gy);
+        if (fi < N) lap = lap6(c0, e, w, n, s, ne, nw, se, sw);
+    }
+    __device__ __forceinline__ V f(int i) const { return ld.template pop_late<KIND_F>(0, i, oc, 5); }
+    __device__ __forceinline__ V g(int p, int i) const { return ld.template pop_late<KIND_G>(1 + p, i, oc, 6); }
+    __device__ __forceinline__ V h(int i) const { return ld.template pop_late<KIND_H>(N + 1, i, oc, 7); }
     __device__ __forceinline__ V lag(int a) const { return ld.aux(a, oc, 14); }
     template <int KIND>
     __device__ __forceinline__ void push(int s, const V (&q)[9])
@@ -357,29 +368,46 @@ struct CellIo {
     // post-collision population is h_eq(ghost) + (1 - 1/tau_h)(h_j - h_eq_j) for the
     // three directions j that enter the boundary row (one code path for both walls:
     // directions (0, sy), (1, sy), (-1, sy), sy = +1 at the bottom, -1 at the top).
-    // Populations, Z and E in their stored form (SCALED: over w_j and rho_ref c_p,ref).
+    __device__ __forceinline__ int dirichlet_side() const
+    {
+        return (y == 0 && P.bc[2] == WALL && P.tbc[2] == DIRICHLET)          ? 2
+               : (y == P.ny - 1 && P.bc[3] == WALL && P.tbc[3] == DIRICHLET) ? 3
+                                                                             : -1;
+    }
     __device__ __forceinline__ void dirichlet(const V (&h)[9], V oh1, V Z, V E, V T, V ux, V uy, V uu)
     {
         using K = exact_t<V>;
-        const int side = (y == 0 && P.bc[2] == WALL && P.tbc[2] == DIRICHLET)             ? 2
-                         : (y == P.ny - 1 && P.bc[3] == WALL && P.tbc[3] == DIRICHLET) ? 3
-                                                                                        : -1;
+        const int side = dirichlet_side();
         if (side < 0) return;
         const auto& C = coef<const_t<V>>(P);
         const bool top = side == 3;
         const V vy = top ? -uy : uy;
-        V Eg = V(C.Tw[side]) * K(2) - T;
-        if constexpr (!Pr::QUANT) Eg = Eg * C.E_ref;
+        const V Eg = (V(C.Tw[side]) * K(2) - T) * C.E_ref;
         const V uu15 = uu * K(-1.5);
         // equilibrium (over w_j) of a moving direction with c_j . u = cu
         auto heq = [&](V cu) { return rfma(Z, rfma(cu * K(4.5), cu, rfma(cu, K(3), uu15)), E); };
-        auto value = [&](V hj, V cu, int j) {
-            if constexpr (Pr::QUANT) return rfma(oh1, hj - heq(cu), Eg);
-            else return rfma(oh1, hj - heq(cu) * wgt_v<V>(j), Eg * wgt_v<V>(j));
-        };
+        auto value = [&](V hj, V cu, int j) { return rfma(oh1, hj - heq(cu) * wgt_v<V>(j), Eg * wgt_v<V>(j)); };
         push_row_at<KIND_H, Pr>(P, pout, N + 1, top ? 4 : 2, 0, x, y, value(top ? h[4] : h[2], vy, 2));
         push_row_at<KIND_H, Pr>(P, pout, N + 1, top ? 8 : 5, 1, x, y, value(top ? h[8] : h[5], ux + vy, 5));
         push_row_at<KIND_H, Pr>(P, pout, N + 1, top ? 7 : 6, -1, x, y, value(top ? h[7] : h[6], vy - ux, 5));
+    }
+    // The same in the order of roundings that 16-bit storage keeps (lbm_cell16.cuh).
+    __device__ __forceinline__ void dirichlet16(const float (&h)[9], float oh1, float Z, float E, float T, float ux, float uy,
+                                                float uu)
+    {
+        const int side = dirichlet_side();
+        if (side < 0) return;
+        const Coef<float>& C = P.f;
+        const bool top = side == 3;
+        const float vy = top ? -uy : uy;
+        const float Eg = C.E_ref * (2.0f * C.Tw[side] - T);
+        auto heq = [&](float w, float cu) { return w * rfma(Z, rfma(4.5f * cu, cu, rfma(3.0f, cu, -1.5f * uu)), E); };
+        const float wa = wgt_r<float>(2), wd = wgt_r<float>(5);
+        push_row_at<KIND_H, Pr>(P, pout, N + 1, top ? 4 : 2, 0, x, y, rfma(oh1, (top ? h[4] : h[2]) - heq(wa, vy), wa * Eg));
+        push_row_at<KIND_H, Pr>(P, pout, N + 1, top ? 8 : 5, 1, x, y,
+                                rfma(oh1, (top ? h[8] : h[5]) - heq(wd, ux + vy), wd * Eg));
+        push_row_at<KIND_H, Pr>(P, pout, N + 1, top ? 7 : 6, -1, x, y,
+                                rfma(oh1, (top ? h[7] : h[6]) - heq(wd, vy - ux), wd * Eg));
     }
     __device__ __forceinline__ void put_fields(const V (&phi)[N], V T, V H_, V fl, V ux, V uy, V p)
     {
@@ -454,7 +482,7 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
                                             typename Pr::TA* __restrict__ aout, const ExportPtrs& ex, int bx, int by,
                                             typename Pr::R* smem)
 {
-    using V = val_t<typename Pr::R>;
+    using V = step_val<Pr>;
     constexpr int W = TX + 2, H = TY + 2, CELLS = TX * TY, NT = RING_TEAM ? 2 * CELLS : CELLS;
     V* fields = reinterpret_cast<V*>(smem);
     V (*s_phi)[H][W] = reinterpret_cast<V (*)[H][W]>(fields);          // [N][H][W]
@@ -497,15 +525,19 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
         }
     };
     // phi_p, rho and psi of a position to shared memory
-    auto share = [&](int lx, int ly, const V (&ph)[N], V fl) {
-        V r, ps;
-        mix_rho_psi<N>(P, ph, fl, r, ps);
+    auto put = [&](int lx, int ly, const V (&ph)[N], V r, V ps) {
 #pragma unroll
         for (int p = 0; p < N; ++p) s_phi[p][ly][lx] = ph[p];
         s_rho[ly][lx] = r;
         s_psi[ly][lx] = ps;
     };
+    auto share = [&](int lx, int ly, const V (&ph)[N], V fl) {
+        V r, ps;
+        mix_rho_psi<N>(P, ph, fl, r, ps);
+        put(lx, ly, ph, r, ps);
+    };
     V phi[N], rhoH, fl;
+    Cell16<N> m;   // 16-bit storage
     if constexpr (Pr::COMPACT) {
         // ---- stages A + B: one code path for all (TX + 2)(TY + 2) positions, so that
         // the moments are compiled once; the own cells' rho H and f_l go to shared memory
@@ -529,13 +561,24 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
         auto halo_at = [&](int lx, int ly) {
             Cell cell;
             if (!locate(lx, ly, cell)) return;
-            V ph[N], rH, flv;
-            cell_moments<N, Pr>(P, ld, cell, ph, rH, flv);
-            share(lx, ly, ph, flv);
+            if constexpr (Pr::QUANT) {
+                Cell16<N> r;
+                moments16<N, false>(P, ld, cell, r);
+                put(lx, ly, r.phi, r.rho, r.psi);
+            } else {
+                V ph[N], rH, flv;
+                cell_moments<N, Pr>(P, ld, cell, ph, rH, flv);
+                share(lx, ly, ph, flv);
+            }
         };
         if (owned) {
-            cell_moments<N, Pr>(P, ld, ld.own(x, y, tx, ty), phi, rhoH, fl);
-            share(tx + 1, ty + 1, phi, fl);
+            if constexpr (Pr::QUANT) {
+                moments16<N, true>(P, ld, ld.own(x, y, tx, ty), m);
+                put(tx + 1, ty + 1, m.phi, m.rho, m.psi);
+            } else {
+                cell_moments<N, Pr>(P, ld, ld.own(x, y, tx, ty), phi, rhoH, fl);
+                share(tx + 1, ty + 1, phi, fl);
+            }
         } else if (own_team) {
             halo_at(tx + 1, ty + 1);
         }
@@ -569,7 +612,8 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
     const PopView<Pr> pout = pop_view<Pr>(P, pout_base);
     CellIo<N, H, W, Pr, L> io{P, ld, fields, pout, aout, ex, tx + 1, ty + 1, x, y, inside, (unsigned)y * (unsigned)nx + (unsigned)x,
                               ld.own(x, y, tx, ty)};
-    cell_update<N, COLLIDE, Pr>(P, io, phi, rhoH, fl);
+    if constexpr (Pr::QUANT) cell_update16<N, COLLIDE, Pr>(P, io, m);
+    else cell_update<N, COLLIDE, Pr>(P, io, phi, rhoH, fl);
 }
 
 // One TX x TY tile read from global memory (the loader of the one-cell step).

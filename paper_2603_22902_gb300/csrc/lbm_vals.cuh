@@ -74,6 +74,7 @@ using val_t = typename std::conditional<std::is_same<R, float>::value, f1,
 // would run on the 2-lane FP64 unit; magnitudes below FP32's normal range become 0 (or a value
 // below 2^-126), magnitudes above it, infinities and NaN become infinite.
 __device__ __forceinline__ float lead(f1 a) { return a.v; }
+__device__ __forceinline__ float lead(float a) { return a; }
 __device__ __forceinline__ float lead(df64 a) { return a.hi; }
 __device__ __forceinline__ float lead(d1 a)
 {
