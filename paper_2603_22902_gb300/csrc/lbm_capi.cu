@@ -279,7 +279,6 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
     P.d.omega_g1 = 1.0 - P.d.omega_g;
     const double gc[3] = {3.0 * (P.d.omega_g + P.d.kg), -3.0 * P.d.kg, P.d.kg};
     for (int k = 0; k < 3; ++k) P.d.g_pl[k] = gc[k] / 9.0;
-    P.ordered = th->T_sol <= 0.0 && th->T_liq >= 0.0 ? 1 : 0;
 
     const size_t pb = plane_bytes(h);
     P.rest_elems = (long long)(N + 2) * P.S;

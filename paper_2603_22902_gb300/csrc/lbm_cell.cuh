@@ -119,13 +119,13 @@ __device__ __forceinline__ V phi_sum(const V (&phi)[N], const C (&a)[MAXN])
     return v;
 }
 
-// The FP32 screen of eq. H for one cell: 1 (liquid) where rho H lies above the liquidus value Al, 0
-// (solid) where phase-changing material is present and rho H lies below the solidus value As, by
-// more than 1e-5 of the magnitudes involved: at least ten times the rounding of As and Al from
-// leading parts; -1 where it does not decide (the mushy band, values near a threshold,
-// phase-changing material below FP32 range, values that are not finite).  Where the solidus
-// value can lie above the liquidus value (P.ordered = 0), a liquid cell has to clear both, as
-// in the map.
+// The FP32 screen of eq. H for one cell: 1 (liquid) where rho H lies above the liquidus value Al (and
+// the solidus value As), 0 (solid) where phase-changing material is present (Lv > 0) and rho H lies
+// below As, -1 where it does not decide (the mushy band, values near a threshold, phase-changing
+// material below FP32 range or whose fractions cancel, values that are not finite).  Al, As and Lv are
+// sums over the phases, and the tails of absent phases have either sign: the margin is 1e-5 of the
+// sums of magnitudes, which is at least ten times the rounding of Al and As from leading parts, and Lv
+// counts as positive or negative only beyond 1e-5 of its own.  With T_sol = T_liq = 0 Al is Lv and As is 0.
 template <int N, class V>
 __device__ __forceinline__ int eqh_screen(const KParams& P, const V (&phi)[N], V rhoH)
 {
@@ -134,27 +134,39 @@ __device__ __forceinline__ int eqh_screen(const KParams& P, const V (&phi)[N], V
 #pragma unroll
     for (int p = 0; p < N; ++p) ph[p] = lead(phi[p]);
     const float h = lead(rhoH);
-    float rl = __fmul_rn(ph[0], C.rho_l[0]), cl = __fmul_rn(ph[0], C.cp_l[0]), Lv = __fmul_rn(ph[0], C.rhoL[0]);
+    float Lv = __fmul_rn(ph[0], C.rhoL[0]), La = fabsf(Lv);
 #pragma unroll
     for (int p = 1; p < N; ++p) {
-        rl = __fmaf_rn(ph[p], C.rho_l[p], rl);
-        cl = __fmaf_rn(ph[p], C.cp_l[p], cl);
         Lv = __fmaf_rn(ph[p], C.rhoL[p], Lv);
+        La = __fmaf_rn(fabsf(ph[p]), C.rhoL[p], La);
     }
-    const float Ac = __fmul_rn(__fmul_rn(rl, cl), C.T_liq), Al = __fadd_rn(Ac, Lv);
-    const float tol = __fmaf_rn(1e-5f, __fadd_rn(__fadd_rn(fabsf(Ac), fabsf(Lv)), fabsf(h)), 1e-30f);
-    const bool above = h > __fadd_rn(Al, tol);
-    if (above && P.ordered) return 1;
-    float rs = __fmul_rn(ph[0], C.rho_s[0]), cs = __fmul_rn(ph[0], C.cp_s[0]);
+    float Al = Lv, As = 0.0f, mag = __fadd_rn(La, fabsf(h));
+    const bool shifted = C.T_liq != 0.0f || C.T_sol != 0.0f;
+    if (shifted) {
+        float rl = 0.0f, cl = 0.0f, rs = 0.0f, cs = 0.0f, rla = 0.0f, cla = 0.0f, rsa = 0.0f, csa = 0.0f;
 #pragma unroll
-    for (int p = 1; p < N; ++p) {
-        rs = __fmaf_rn(ph[p], C.rho_s[p], rs);
-        cs = __fmaf_rn(ph[p], C.cp_s[p], cs);
+        for (int p = 0; p < N; ++p) {
+            const float a = fabsf(ph[p]);
+            rl = __fmaf_rn(ph[p], C.rho_l[p], rl);
+            cl = __fmaf_rn(ph[p], C.cp_l[p], cl);
+            rs = __fmaf_rn(ph[p], C.rho_s[p], rs);
+            cs = __fmaf_rn(ph[p], C.cp_s[p], cs);
+            rla = __fmaf_rn(a, C.rho_l[p], rla);
+            cla = __fmaf_rn(a, C.cp_l[p], cla);
+            rsa = __fmaf_rn(a, C.rho_s[p], rsa);
+            csa = __fmaf_rn(a, C.cp_s[p], csa);
+        }
+        Al = __fmaf_rn(__fmul_rn(rl, cl), C.T_liq, Lv);
+        As = __fmul_rn(__fmul_rn(rs, cs), C.T_sol);
+        mag = __fmaf_rn(__fmul_rn(rla, cla), fabsf(C.T_liq), mag);
+        mag = __fmaf_rn(__fmul_rn(rsa, csa), fabsf(C.T_sol), mag);
     }
-    const float As = __fmul_rn(__fmul_rn(rs, cs), C.T_sol);
-    const float tols = __fmaf_rn(1e-5f, fabsf(As), tol);
-    if (above && h > __fadd_rn(As, tols)) return 1;
-    if (Lv > 0.0f && h < __fsub_rn(As, tols)) return 0;
+    const float tol = __fmaf_rn(1e-5f, mag, 1e-30f);
+    // without phase-changing material a cell is liquid whatever As; with it and As = 0 (not shifted), above Al is above As
+    if (h > __fadd_rn(Al, tol) && (!shifted || h > __fadd_rn(As, tol) || Lv < __fmul_rn(-1e-5f, La))) return 1;
+    // a double's leading part is 0 below 2^-126
+    const float none = std::is_same<V, d1>::value ? 1e-30f : 0.0f;
+    if (Lv > __fmaf_rn(1e-5f, La, none) && h < __fsub_rn(As, tol)) return 0;
     return -1;
 }
 

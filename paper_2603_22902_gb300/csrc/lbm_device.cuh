@@ -64,9 +64,8 @@ struct Coef {
 // Everything derivable once per run is derived on the host.
 struct KParams {
     int nx, ny, N;
+    unsigned S32;                 // S as 32 bits; a lattice whose sets fit this GPU has fewer than 2^30 cells
     long long S;                  // plane stride in elements (nx * ny)
-    unsigned S32;                 // the same; a lattice whose sets fit this GPU has fewer than 2^30 cells
-    int ordered;                  // 1: T_sol <= 0 <= T_liq, so As <= Al - Lv in eq. H
     int bc[4], tbc[4];            // side kinds, sides 0 x-min, 1 x-max, 2 y-min, 3 y-max
     Coef<double> d;               // coefficients, FP64
     Coef<float> f;                // the same, rounded to FP32
