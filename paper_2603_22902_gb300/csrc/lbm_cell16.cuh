@@ -94,11 +94,12 @@ __device__ __forceinline__ void cell_update16(const KParams& P, Io& io, const Ce
     float gpx[N + 2], gpy[N + 2], lap[N];
 #pragma unroll
     for (int fi = 0; fi < N + 2; ++fi) {
-        float v0, e, w, n, s, ne, nw, se, sw;
-        io.window(fi, v0, e, w, n, s, ne, nw, se, sw);
+        const float e = io.at(fi, 1, 0), w = io.at(fi, -1, 0), n = io.at(fi, 0, 1), s = io.at(fi, 0, -1);
+        const float ne = io.at(fi, 1, 1), nw = io.at(fi, -1, 1), se = io.at(fi, 1, -1), sw = io.at(fi, -1, -1);
         gpx[fi] = (e - w) * float(1.0 / 3.0) + ((ne - nw) + (se - sw)) * float(1.0 / 12.0);
         gpy[fi] = (n - s) * float(1.0 / 3.0) + ((ne - se) + (nw - sw)) * float(1.0 / 12.0);
         if (fi < N) {
+            const float v0 = io.at(fi, 0, 0);
             const float ax = (e + w) + (n + s);
             const float dg = (ne + nw) + (se + sw);
             lap[fi] = ax * float(2.0 / 3.0) + dg * float(1.0 / 6.0) - v0 * float(10.0 / 3.0);

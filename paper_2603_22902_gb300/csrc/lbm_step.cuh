@@ -336,20 +336,18 @@ struct CellIo {
     bool inside;                   // push_species
     unsigned c;
     typename L::Cell oc;
-    // the nine values of field fi around the cell
-    __device__ __forceinline__ void window(int fi, V& c0, V& e, V& w, V& n, V& s, V& ne, V& nw, V& se, V& sw) const
+    // the values of field fi at offset (dx, dy) from the cell
+    __device__ __forceinline__ V at(int fi, int dx, int dy) const
     {
-        const V (*a)[W] = reinterpret_cast<const V (*)[W]>(fields + fi * H * W);
-        e = a[ly][lx + 1], w = a[ly][lx - 1], n = a[ly + 1][lx], s = a[ly - 1][lx];
-        ne = a[ly + 1][lx + 1], nw = a[ly + 1][lx - 1], se = a[ly - 1][lx + 1], sw = a[ly - 1][lx - 1];
-        if (fi < N) c0 = a[ly][lx];
+        return reinterpret_cast<const V (*)[W]>(fields + fi * H * W)[ly + dy][lx + dx];
     }
     __device__ __forceinline__ void stencil(int fi, V& gx, V& gy, V& lap) const
     {
-        V c0, e, w, n, s, ne, nw, se, sw;
-        window(fi, c0, e, w, n, s, ne, nw, se, sw);
+        const V (*a)[W] = reinterpret_cast<const V (*)[W]>(fields + fi * H * W);
+        const V e = a[ly][lx + 1], w = a[ly][lx - 1], n = a[ly + 1][lx], s = a[ly - 1][lx];
+        const V ne = a[ly + 1][lx + 1], nw = a[ly + 1][lx - 1], se = a[ly - 1][lx + 1], sw = a[ly - 1][lx - 1];
         grad12(e, w, n, s, ne, nw, se, sw, gx, gy);
-        if (fi < N) lap = lap6(c0, e, w, n, s, ne, nw, se, sw);
+        if (fi < N) lap = lap6(a[ly][lx], e, w, n, s, ne, nw, se, sw);
     }
     __device__ __forceinline__ V f(int i) const { return ld.template pop_late<KIND_F>(0, i, oc, 5); }
     __device__ __forceinline__ V g(int p, int i) const { return ld.template pop_late<KIND_G>(1 + p, i, oc, 6); }
