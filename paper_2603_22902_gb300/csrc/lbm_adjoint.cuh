@@ -157,15 +157,17 @@ __device__ __forceinline__ int eqh_branch(const KParams& P, const double (&phi)[
         return sure;
     }
     const Mix<N> m = mixture_map<N>(P, phi);
-    const double As = m.rs * m.cs * P.T_sol, Al = fma(m.rl * m.cl, P.T_liq, m.Lv);
+    // as enthalpy_map rounds them
+    const double As = __dmul_rn(__dmul_rn(m.rs, m.cs), P.T_sol), Al = __fma_rn(__dmul_rn(m.rl, m.cl), P.T_liq, m.Lv);
+    const double band = __dsub_rn(Al, As);
     fl = 1.0;
     if (!(m.Lv > 0.0) || (!(rhoH < As) && rhoH > Al)) return EQH_LIQUID;
     if (rhoH < As) {
         fl = 0.0;
         return EQH_SOLID;
     }
-    if (!(Al - As > 0.0)) return EQH_POINT;
-    fl = (rhoH - As) / (Al - As);
+    if (!(band > 0.0)) return EQH_POINT;
+    fl = __ddiv_rn(__dsub_rn(rhoH, As), band);
     return EQH_MUSHY;
 }
 

@@ -291,25 +291,28 @@ __device__ __forceinline__ R mix_sum(const R (&phi)[N], const R (&a)[MAXN])
 
 // eq. H: liquid fraction (and, with WANT_T, temperature) from rho H.
 // rho_s H_s = rs cs T_sol, rho_l H_l = rl cl T_liq + Lv; a cell without phase-changing
-// material (Lv <= 0) is liquid (the ambient fluid has f_s = 0).
+// material (Lv <= 0) is liquid (the ambient fluid has f_s = 0).  Every operation is a round-to-nearest
+// intrinsic: products and differences fused by the compiler, here and there in another way, would
+// give a cell other bits in another kernel.
 template <int N, bool WANT_T>
 __device__ __forceinline__ void enthalpy_map(const KParams& P, const Mix<N>& m, double rhoH, double& fl, double& T)
 {
-    const double rcs = m.rs * m.cs, rcl = m.rl * m.cl;
-    const double As = rcs * P.T_sol;
-    const double Al = fma(rcl, P.T_liq, m.Lv);
+    const double rcs = __dmul_rn(m.rs, m.cs), rcl = __dmul_rn(m.rl, m.cl);
+    const double As = __dmul_rn(rcs, P.T_sol);
+    const double Al = __fma_rn(rcl, P.T_liq, m.Lv), band = __dsub_rn(Al, As);
+    auto liquid_T = [&] { return __dadd_rn(P.T_liq, __ddiv_rn(__dsub_rn(rhoH, Al), rcl)); };
     if (!(m.Lv > 0.0)) {
         fl = 1.0;
-        if (WANT_T) T = P.T_liq + (rhoH - Al) / rcl;
+        if (WANT_T) T = liquid_T();
     } else if (rhoH < As) {
         fl = 0.0;
-        if (WANT_T) T = rhoH / rcs;
+        if (WANT_T) T = __ddiv_rn(rhoH, rcs);
     } else if (rhoH > Al) {
         fl = 1.0;
-        if (WANT_T) T = P.T_liq + (rhoH - Al) / rcl;
-    } else if (Al - As > 0.0) {
-        fl = (rhoH - As) / (Al - As);
-        if (WANT_T) T = fma(fl, P.T_liq - P.T_sol, P.T_sol);
+        if (WANT_T) T = liquid_T();
+    } else if (band > 0.0) {
+        fl = __ddiv_rn(__dsub_rn(rhoH, As), band);
+        if (WANT_T) T = __fma_rn(fl, __dsub_rn(P.T_liq, P.T_sol), P.T_sol);
     } else {
         fl = 1.0;
         if (WANT_T) T = P.T_liq;
@@ -320,13 +323,12 @@ __device__ __forceinline__ void enthalpy_map(const KParams& P, const Mix<N>& m, 
 template <int N>
 __device__ __forceinline__ double inverse_map(const KParams& P, const Mix<N>& m, double T)
 {
-    const double rcs = m.rs * m.cs, rcl = m.rl * m.cl;
-    const double As = rcs * P.T_sol;
-    const double Al = fma(rcl, P.T_liq, m.Lv);
-    if (!(m.Lv > 0.0)) return Al + rcl * (T - P.T_liq);
-    if (T < P.T_sol) return rcs * T;
-    if (T >= P.T_liq) return Al + rcl * (T - P.T_liq);
-    return As + (T - P.T_sol) / (P.T_liq - P.T_sol) * (Al - As);
+    const double rcs = __dmul_rn(m.rs, m.cs), rcl = __dmul_rn(m.rl, m.cl);
+    const double Al = __fma_rn(rcl, P.T_liq, m.Lv);
+    if (!(m.Lv > 0.0) || T >= P.T_liq) return __fma_rn(rcl, __dsub_rn(T, P.T_liq), Al);
+    if (T < P.T_sol) return __dmul_rn(rcs, T);
+    const double As = __dmul_rn(rcs, P.T_sol);
+    return __fma_rn(__ddiv_rn(__dsub_rn(T, P.T_sol), __dsub_rn(P.T_liq, P.T_sol)), __dsub_rn(Al, As), As);
 }
 
 // g'(x) for g(x) = x^2 (1 - x)^2
