@@ -98,7 +98,7 @@ batch_persistent_kernel(const BatchTable T, int nsteps)
             }
             const BatchCase& C = T.cases[c];
             const int local = t - C.first_tile;
-            step_tile<N, TX, TY, true, PC>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
+            step_tile<N, TX, TY, true, PC, false, true>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
                                            (TA*)C.aux[a ^ 1], ExportPtrs{}, local % C.tiles_x, local / C.tiles_x,
                                            smem);
         }
@@ -123,7 +123,7 @@ batch_step_kernel(const BatchTable T, int s)
     const int a = (*(volatile unsigned char*)T.parity) ^ (s & 1);
     const BatchCase& C = T.cases[c];
     const int local = t - C.first_tile;
-    step_tile<N, TX, TY, true, Pr>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
+    step_tile<N, TX, TY, true, Pr, false, true>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
                                    (TA*)C.aux[a ^ 1], ExportPtrs{}, local % C.tiles_x, local / C.tiles_x, smem);
 }
 
@@ -150,7 +150,7 @@ batch_substep_kernel(const BatchTable T, int s)
     load_params(sP, T.params + c);
     __syncthreads();
     const int a = (*(volatile unsigned char*)T.parity) ^ (s & 1);
-    step_tile<N, 8, 4, true, Pr, RING_TEAM>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
+    step_tile<N, 8, 4, true, Pr, RING_TEAM, true>(sP, C.pop[a], const_cast<void*>(C.pop[a ^ 1]), (const TA*)C.aux[a],
                                  (TA*)C.aux[a ^ 1], ExportPtrs{}, bx, by, smem);
 }
 

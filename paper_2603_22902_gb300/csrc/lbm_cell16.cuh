@@ -83,6 +83,31 @@ __device__ __forceinline__ void moments16(const KParams& P, const L& ld, typenam
     }
 }
 
+// g'(x) - g'(s) of the chemical potentials, g'(x) = A(x) B(x) with A = 2 x (1 - x), B = 1 - 2 x.  The
+// difference can be fused with either product or with none, which rounds in three ways, and a unit in
+// the last place of mu_p is one of u.  The results of these policies were made with the choices below, for
+// term 2 k (phase p) and 2 k + 1 (phase q) of the k-th pair, which the compiler made for each kernel when
+// they were left to it; they are written out so that it makes no others.
+constexpr int FUSE_X = 0, FUSE_S = 1, FUSE_NONE = 2;
+enum Caller16 { CALLER_STEP, CALLER_STAGED, CALLER_BATCH, CALLER_FIELDS };
+template <int N, int CALLER>
+__device__ __forceinline__ constexpr int gdiff_form(int term)
+{
+    if (CALLER == CALLER_STAGED && N == 3) return FUSE_S;
+    if (CALLER == CALLER_FIELDS && N == 4) return FUSE_S;
+    if (CALLER == CALLER_STEP && N == 3 && term < 2) return FUSE_S;
+    if (CALLER == CALLER_STEP && N == 4 && term == 0) return FUSE_NONE;
+    return FUSE_X;
+}
+__device__ __forceinline__ float gdiff(int form, float x, float s)
+{
+    auto A = [](float a) { return __fmul_rn(__fmul_rn(2.0f, a), __fsub_rn(1.0f, a)); };
+    auto B = [](float a) { return __fmaf_rn(-2.0f, a, 1.0f); };
+    if (form == FUSE_X) return __fmaf_rn(A(x), B(x), -__fmul_rn(A(s), B(s)));
+    const float gx = __fmul_rn(A(x), B(x));
+    return form == FUSE_S ? __fmaf_rn(-A(s), B(s), gx) : __fsub_rn(gx, __fmul_rn(A(s), B(s)));
+}
+
 // Stages C to G (see cell_update in lbm_cell.cuh for what io supplies and takes).
 template <int N, bool COLLIDE, class Pr, class Io>
 __device__ __forceinline__ void cell_update16(const KParams& P, Io& io, const Cell16<N>& m)
@@ -109,13 +134,14 @@ __device__ __forceinline__ void cell_update16(const KParams& P, Io& io, const Ce
 
     // ---- stage D: pairwise normals, R_p, chemical potentials, F_s -----------
     const float (&phi)[N] = m.phi;
-    float Rx[N], Ry[N], mup[N], gpv[N];
+    constexpr int CALLER = COLLIDE ? Io::CALLER : CALLER_FIELDS;
+    float Rx[N], Ry[N], mup[N];
+    int term = 0;
 #pragma unroll
     for (int p = 0; p < N; ++p) {
         Rx[p] = 0.0f;
         Ry[p] = 0.0f;
         mup[p] = 0.0f;
-        gpv[p] = 2.0f * phi[p] * (1.0f - phi[p]) * (1.0f - 2.0f * phi[p]);  // g'(phi), g = phi^2 (1 - phi)^2
     }
 #pragma unroll
     for (int p = 0; p < N; ++p)
@@ -142,9 +168,8 @@ __device__ __forceinline__ void cell_update16(const KParams& P, Io& io, const Ce
             Ry[p] = rfma(a, nyv, Ry[p]);
             Rx[q] = rfma(-a, nxv, Rx[q]);
             Ry[q] = rfma(-a, nyv, Ry[q]);
-            const float gs = 2.0f * s * (1.0f - s) * (1.0f - 2.0f * s);
-            mup[p] += rfma(C.b2[p][q], gpv[p] - gs, C.kk[p][q] * lap[q]);
-            mup[q] += rfma(C.b2[q][p], gpv[q] - gs, C.kk[q][p] * lap[p]);
+            mup[p] += rfma(C.b2[p][q], gdiff(gdiff_form<N, CALLER>(term++), phi[p], s), C.kk[p][q] * lap[q]);
+            mup[q] += rfma(C.b2[q][p], gdiff(gdiff_form<N, CALLER>(term++), phi[q], s), C.kk[q][p] * lap[p]);
         }
     float Fx = rho * C.accel[0], Fy = rho * C.accel[1];
 #pragma unroll

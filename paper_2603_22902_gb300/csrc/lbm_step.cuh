@@ -322,8 +322,9 @@ __host__ __device__ constexpr int tile_smem_elems()
 // What cell_update and cell_update16 read and write of the cell (x, y) of a tile: its stencil
 // windows from shared memory (fields of H x W values, the cell at (lx, ly)), its populations and
 // lagged values through the loader, its outputs to set B.
-template <int N, int H, int W, class Pr, class L>
+template <int N, int H, int W, class Pr, class L, bool BATCH = false>
 struct CellIo {
+    static constexpr int CALLER = !L::GLOBAL ? CALLER_STAGED : BATCH ? CALLER_BATCH : CALLER_STEP;
     using V = step_val<Pr>;
     using TA = typename Pr::TA;
     const KParams& P;
@@ -475,7 +476,8 @@ __device__ __forceinline__ void fill_ghosts(const KParams& P, V* fields, int x0,
 // Every thread of the block must call it (it holds two block barriers); the caller
 // places a block barrier before smem is used again.  RING_TEAM: a block of 2 TX TY threads, whose
 // second half evaluates the ring while the first evaluates the tile's cells (not for COMPACT policies).
-template <int N, int TX, int TY, bool COLLIDE, class Pr, bool RING_TEAM = false, class L>
+// BATCH: the caller is a batch's kernel (gdiff_form, lbm_cell16.cuh).
+template <int N, int TX, int TY, bool COLLIDE, class Pr, bool RING_TEAM = false, bool BATCH = false, class L>
 __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void* __restrict__ pout_base,
                                             typename Pr::TA* __restrict__ aout, const ExportPtrs& ex, int bx, int by,
                                             typename Pr::R* smem)
@@ -608,21 +610,21 @@ __device__ __forceinline__ void step_tile_l(const KParams& P, const L& ld, void*
     // side that is not periodic, take the general path
     const bool inside = y >= 1 && y <= ny - 2 && (xper || (x0 >= 1 && x0 + TX <= nx - 1));
     const PopView<Pr> pout = pop_view<Pr>(P, pout_base);
-    CellIo<N, H, W, Pr, L> io{P, ld, fields, pout, aout, ex, tx + 1, ty + 1, x, y, inside, (unsigned)y * (unsigned)nx + (unsigned)x,
+    CellIo<N, H, W, Pr, L, BATCH> io{P, ld, fields, pout, aout, ex, tx + 1, ty + 1, x, y, inside, (unsigned)y * (unsigned)nx + (unsigned)x,
                               ld.own(x, y, tx, ty)};
     if constexpr (Pr::QUANT) cell_update16<N, COLLIDE, Pr>(P, io, m);
     else cell_update<N, COLLIDE, Pr>(P, io, phi, rhoH, fl);
 }
 
 // One TX x TY tile read from global memory (the loader of the one-cell step).
-template <int N, int TX, int TY, bool COLLIDE, class Pr, bool RING_TEAM = false>
+template <int N, int TX, int TY, bool COLLIDE, class Pr, bool RING_TEAM = false, bool BATCH = false>
 __device__ __forceinline__ void step_tile(const KParams& P, const void* __restrict__ pin_base,
                                           void* __restrict__ pout_base, const typename Pr::TA* __restrict__ ain,
                                           typename Pr::TA* __restrict__ aout, const ExportPtrs& ex, int bx, int by,
                                           typename Pr::R* smem)
 {
     const GlobalLoader<Pr> ld{P, pop_view<Pr>(P, pin_base), ain};
-    step_tile_l<N, TX, TY, COLLIDE, Pr, RING_TEAM>(P, ld, pout_base, aout, ex, bx, by, smem);
+    step_tile_l<N, TX, TY, COLLIDE, Pr, RING_TEAM, BATCH>(P, ld, pout_base, aout, ex, bx, by, smem);
 }
 
 // Tile (bx, by) of block b of a one-dimensional grid of tx * ty tiles.  The tiles on the

@@ -35,3 +35,26 @@ def test_run_is_the_recorded_one(prec, name, form):
     with np.load(GOLDEN) as want:
         for k in ("phi", "T", "ux", "uy"):
             assert np.array_equal(F[k].astype(np.float32), want[f"{prec}.{name}.{k}"]), k
+
+
+PHASES = os.path.join(os.path.dirname(__file__), "golden", "storage16_runs_phases.npz")
+MORE = {   # three and four phases: case, options, 20 steps; the one-launch and the staged form have recordings of their own
+    "janus": (lambda: W.perturbed(W.janus_drop(nx=60, ny=33, R=13.0, mobility=0.1), seed=7, amp_u=1e-3, amp_T=0.02), {}),
+    "pool": (lambda: W.perturbed(W.lateral_pool(n=48), seed=7, amp_u=1e-3), dict(staged=False)),
+    "pool_staged": (lambda: W.perturbed(W.lateral_pool(n=48), seed=7, amp_u=1e-3), dict(staged=True)),
+    "impurity": (lambda: W.perturbed(W.impurity_freeze(n=65, n_disks=2), seed=7, amp_u=1e-3, amp_T=0.02), {}),
+}
+
+
+@pytest.mark.parametrize("name", list(MORE))
+@pytest.mark.parametrize("prec", ["bf16s", "fp16s"])
+def test_run_of_more_phases_is_the_recorded_one(prec, name):
+    from paper_2603_22902_gb300 import lbm as L
+    case, options = MORE[name]
+    s = L.Solver(case(), precision=prec, **options).set_fields()
+    s.step(20)
+    F = s.fields_numpy()
+    s.close()
+    with np.load(PHASES) as want:
+        for k in ("ux", "uy"):
+            assert np.array_equal(F[k].astype(np.float32), want[f"{prec}.{name}.{k}"]), k
