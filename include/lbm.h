@@ -377,7 +377,9 @@ typedef struct lbm_batch lbm_batch;
 
 #define LBM_BATCH_PERSISTENT 0 /* one cooperative launch per tile-shape group and call;
                                   grid barrier between steps */
-#define LBM_BATCH_PER_STEP 1   /* one launch per tile-shape group and step */
+#define LBM_BATCH_PER_STEP 1   /* one launch per tile-shape group and step; a 32x8-tile group
+                                  of an LBM_FP64 batch that fills the GPU badly runs on
+                                  smaller tiles (the other shapes are used as they are) */
 #define LBM_BATCH_STAGED 2     /* the per-step form, with every tile of a 32x8-tile group
                                   computed from a TMA-staged copy of its inputs (the staged
                                   step of lbm_set_staging) where the group allows it: policy

@@ -195,10 +195,10 @@ cudaError_t batch_blocks_per_sm(int kind, int* out)
 }
 
 template <int N, int TX, int TY, class Pr>
-static cudaError_t launch_batch_step_t(const BatchTable& T, int s, cudaStream_t st)
+static cudaError_t launch_batch_step_t(const BatchTable& T, int kind, int s, cudaStream_t st)
 {
-    if constexpr (std::is_same<Pr, PrecFP64>::value) {
-        if (fp64_small_tiles(T.total_tiles, T.total_subtiles, T.sms)) {
+    if constexpr (std::is_same<Pr, PrecFP64>::value && TX == 32) {
+        if (fp64_batch_subtiles(kind, T.total_tiles, T.total_subtiles, T.sms)) {
             const bool team = fp64_ring_team(T.total_subtiles, T.sms);
             const auto kernel = team ? batch_substep_kernel<N, TX, TY, Pr, true> : batch_substep_kernel<N, TX, TY, Pr, false>;
             kernel<<<T.total_tiles * BATCH_SUB, BATCH_NT / BATCH_SUB * (team ? 2 : 1), 0, st>>>(T, s);
@@ -214,12 +214,12 @@ cudaError_t launch_batch_step(const BatchTable& T, int kind, int s, cudaStream_t
 {
     if constexpr (single_shape<Pr>()) {
         if (kind != TILE_32x8) return cudaErrorNotSupported;
-        return launch_batch_step_t<N, 32, 8, Pr>(T, s, st);
+        return launch_batch_step_t<N, 32, 8, Pr>(T, kind, s, st);
     } else {
         switch (kind) {
-            case TILE_64x4: return launch_batch_step_t<N, 64, 4, Pr>(T, s, st);
-            case TILE_16x16: return launch_batch_step_t<N, 16, 16, Pr>(T, s, st);
-            default: return launch_batch_step_t<N, 32, 8, Pr>(T, s, st);
+            case TILE_64x4: return launch_batch_step_t<N, 64, 4, Pr>(T, kind, s, st);
+            case TILE_16x16: return launch_batch_step_t<N, 16, 16, Pr>(T, kind, s, st);
+            default: return launch_batch_step_t<N, 32, 8, Pr>(T, kind, s, st);
         }
     }
 }

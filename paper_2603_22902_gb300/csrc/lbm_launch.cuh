@@ -48,6 +48,12 @@ inline bool fp64_small_tiles(long long tiles, long long subtiles, int sms)
 // Measured, us per step, one warp / two: film 16 x 256 23.8 / 20.1; N = 3, 128^2 30.8 / 28.7; N = 4, 112^2
 // 43.9 / 38.4, 128^2 46.1 / 42.0; beyond four tiles N = 3, 224^2 61.5 / 65.6, 300 x 150 59.4 / 65.6.
 inline bool fp64_ring_team(long long tiles, int sms) { return tiles <= 4LL * sms; }
+// Whether the per-step form of an FP64 batch group cuts its tiles into tiles of 8x4: by the same rule, where
+// the plan has the initial shape, 32x8.  64x4 and 16x16 are in a plan because someone asked for them.
+inline bool fp64_batch_subtiles(int kind, long long tiles, long long subtiles, int sms)
+{
+    return kind == TILE_32x8 && fp64_small_tiles(tiles, subtiles, sms);
+}
 inline int fp64_tile(int nx, int ny, int sms)
 {
     const long long big = (long long)((nx + 31) / 32) * ((ny + 7) / 8), small = (long long)((nx + 7) / 8) * ((ny + 3) / 4);
