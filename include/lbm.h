@@ -135,7 +135,9 @@ typedef struct {
  * with zero diagonal, boundary combinations), derives beta_pq, k_pq and c_p,ref on
  * the host and allocates two population sets of 9 (N + 2) planes and two sets of
  * 3 + 2N lagged planes.  *out is set to NULL on failure.  The state is undefined
- * until lbm_set_fields. */
+ * until lbm_set_fields.
+ * A lattice with a plane of more than 4 GB (2^29 cells of LBM_FP64 or LBM_DF64, 2^30 of the
+ * others) is LBM_EINVAL. */
 int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_thermal* thermal,
                const lbm_bc* bc, const lbm_numerics* numerics, lbm_handle** out);
 

@@ -178,10 +178,12 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
     *out = nullptr;
     if (!grid || !phases || !th || !bc || !num) return fail(nullptr, LBM_EINVAL, "NULL argument");
     if (grid->nx < 3 || grid->ny < 3) return fail(nullptr, LBM_EINVAL, "nx and ny must be >= 3");
-    if ((long long)grid->nx * grid->ny > (1LL << 31)) return fail(nullptr, LBM_EINVAL, "grid too large");
     if (N < 2 || N > LBM_MAXN) return fail(nullptr, LBM_EINVAL, "N must be in [2, 4]");
     if (num->precision < LBM_FP64 || num->precision > LBM_DF64)
         return fail(nullptr, LBM_EINVAL, "precision must be LBM_FP64, LBM_FP32, LBM_FP16S, LBM_BF16S or LBM_DF64");
+    // the kernels address the elements of a plane by 32-bit byte offsets (plane_elem)
+    if ((long long)grid->nx * grid->ny > plane_cells_max(num->precision == LBM_FP64 || num->precision == LBM_DF64 ? 8 : 4))
+        return fail(nullptr, LBM_EINVAL, "grid too large: a plane of more than 4 GB");
     if (!(num->eps > 0.0) || !(num->mobility > 0.0)) return fail(nullptr, LBM_EINVAL, "eps and mobility must be > 0");
     if (num->diag_every < 0) return fail(nullptr, LBM_EINVAL, "diag_every must be >= 0");
     if (!(th->T_sol <= th->T_liq)) return fail(nullptr, LBM_EINVAL, "T_sol must be <= T_liq");

@@ -64,7 +64,7 @@ struct Coef {
 // Everything derivable once per run is derived on the host.
 struct KParams {
     int nx, ny, N;
-    unsigned S32;                 // S as 32 bits; a lattice whose sets fit this GPU has fewer than 2^30 cells
+    unsigned S32;                 // S as 32 bits (plane_cells_max)
     long long S;                  // plane stride in elements (nx * ny)
     int bc[4], tbc[4];            // side kinds, sides 0 x-min, 1 x-max, 2 y-min, 3 y-max
     Coef<double> d;               // coefficients, FP64
@@ -185,10 +185,13 @@ __device__ __forceinline__ T lbm_zero_like(const T*)
 #endif
 #define LBM_LD(P_, ptr, idx, lim, site) LBM_LDX(false, P_, ptr, idx, lim, site)
 
+// Cells of a lattice whose planes of elements of elem_bytes stay within 4 GB, so that 32-bit byte offsets
+// reach them: lbm_create accepts no more.
+__host__ __device__ constexpr long long plane_cells_max(int elem_bytes) { return (1LL << 32) / elem_bytes; }
+
 // Element c of plane `plane` of a block of planes.  The plane's address is the same for all
-// threads; only a 32-bit byte offset is each thread's own (fewer than 2^30 cells, elements of at
-// most 8 bytes and at most 4 GB to a plane: a lattice with more would not fit the memory), so an
-// access costs few integer instructions.  With 64-bit indices per access, a third of the FP32
+// threads; only a 32-bit byte offset is each thread's own (plane_cells_max), so an access costs
+// few integer instructions.  With 64-bit indices per access, a third of the FP32
 // step's instructions were address arithmetic (N = 3: 690 of 1800 per cell, now 436; FP16 storage
 // N = 2: 280 of 1220, now 245); double words at 512^2 went from 65 to 60 us, FP16 storage from 18.7
 // to 17.2 us.
