@@ -171,37 +171,23 @@ __device__ __forceinline__ int eqh_branch(const KParams& P, const double (&phi)[
     return EQH_MUSHY;
 }
 
-// Reverse of eq. H: adjoints (fl_b, T_b) of the outputs -> adjoints of the mixture sums
-// and of rho H, along the branch the forward map takes.
+// Reverse of eq. H in the mushy band, f_l = (rhoH - As) / (Al - As), T = T_sol + f_l (T_liq - T_sol):
+// adjoints (fl_b, T_b) of the outputs -> adjoints of the mixture sums and of rho H.  At EQH_POINT
+// neither depends on them; a cell that is wholly liquid or solid does not come here.
 template <int N>
-__device__ __forceinline__ void map_reverse(const KParams& P, const Mix<N>& m, double rhoH, double fl_b, double T_b,
+__device__ __forceinline__ void map_reverse(const KParams& P, const Mix<N>& m, int branch, double fl, double fl_b, double T_b,
                                             double& rs_b, double& rl_b, double& cs_b, double& cl_b, double& Lv_b,
                                             double& rhoH_b)
 {
+    if (branch != EQH_MUSHY) return;
     const double rcs = m.rs * m.cs, rcl = m.rl * m.cl;
     const double As = rcs * P.T_sol;
     const double Al = fma(rcl, P.T_liq, m.Lv);
-    double rcs_b = 0.0, rcl_b = 0.0, As_b = 0.0, Al_b = 0.0;
-    if (!(m.Lv > 0.0) || (!(rhoH < As) && rhoH > Al)) {
-        // liquid: f_l = 1, T = T_liq + (rhoH - Al) / rcl
-        rhoH_b += T_b / rcl;
-        Al_b -= T_b / rcl;
-        rcl_b -= (rhoH - Al) / (rcl * rcl) * T_b;
-    } else if (rhoH < As) {
-        // solid: f_l = 0, T = rhoH / rcs
-        rhoH_b += T_b / rcs;
-        rcs_b -= rhoH / (rcs * rcs) * T_b;
-    } else if (Al - As > 0.0) {
-        // mushy: f_l = (rhoH - As) / (Al - As), T = T_sol + f_l (T_liq - T_sol)
-        const double d = Al - As;
-        const double fl = (rhoH - As) / d;
-        const double flb = fl_b + T_b * (P.T_liq - P.T_sol);
-        rhoH_b += flb / d;
-        As_b += flb * (fl - 1.0) / d;
-        Al_b -= flb * fl / d;
-    }
-    rcs_b += P.T_sol * As_b;
-    rcl_b += P.T_liq * Al_b;
+    const double d = Al - As;
+    const double flb = fl_b + T_b * (P.T_liq - P.T_sol);
+    rhoH_b += flb / d;
+    const double As_b = flb * (fl - 1.0) / d, Al_b = -(flb * fl / d);
+    const double rcs_b = P.T_sol * As_b, rcl_b = P.T_liq * Al_b;
     Lv_b += Al_b;
     rs_b += m.cs * rcs_b;
     cs_b += m.rs * rcs_b;
@@ -891,7 +877,7 @@ __global__ void __launch_bounds__(ADJ_NT) adj_cell_kernel(const KParams P, const
         const double Ks_b = lam_b * fs, Kl_b = lam_b * fl, Cs_b = cp_b * fs, Cl_b = cp_b * fl;
         const double Dr_b = psi_b * fs, Pc_b = chi_b * fs;
         double rs_b = 0, rl_b = 0, cs_b = 0, cl_b = 0, Lv_b = 0;
-        map_reverse<N>(P, m, rhoH, fl_b, T_b, rs_b, rl_b, cs_b, cl_b, Lv_b, rhoH_b);
+        map_reverse<N>(P, m, branch, fl, fl_b, T_b, rs_b, rl_b, cs_b, cl_b, Lv_b, rhoH_b);
         for (int p = 0; p < N; ++p) {
             phi_b[p] += Rs_b * C.rho_s[p] + Rl_b * C.rho_l[p] + Ms_b * C.mu_s[p] + Ml_b * C.mu_l[p] +
                         Ks_b * C.lam_s[p] + Kl_b * C.lam_l[p] + Cs_b * C.cp_s[p] + Cl_b * C.cp_l[p] +
@@ -1001,7 +987,7 @@ __global__ void __launch_bounds__(ADJ_NT) adj_moments_kernel(const KParams P, co
         fl_b += rho_b * m.rl - fs_b;
         const double Rs_b = rho_b * fs, Rl_b = rho_b * fl, Dr_b = psi_b * fs;
         double rs_b = 0, rl_b = 0, cs_b = 0, cl_b = 0, Lv_b = 0;
-        map_reverse<N>(P, m, rhoH, fl_b, 0.0, rs_b, rl_b, cs_b, cl_b, Lv_b, rhoH_b);
+        map_reverse<N>(P, m, branch, fl, fl_b, 0.0, rs_b, rl_b, cs_b, cl_b, Lv_b, rhoH_b);
         for (int p = 0; p < N; ++p) {
             phi_b[p] += Rs_b * C.rho_s[p] + Rl_b * C.rho_l[p] + Dr_b * C.drho[p];
             phi_b[p] += rs_b * P.d.rho_s[p] + rl_b * P.d.rho_l[p] + cs_b * P.d.cp_s[p] + cl_b * P.d.cp_l[p] +

@@ -151,7 +151,7 @@ struct AdjBufs {
     const double* baux;    // adjoint of set B lagged planes
     double* apop;          // adjoint of set A populations (written)
     double* aaux;          // adjoint of set A lagged planes (written)
-    const double* mac;     // phi_p (N planes), rho, psi of set A
+    const double* mac;     // phi_p (N planes), rho, psi, rho H of set A
     double* own;           // phi_p-bar (N planes) and rhoH-bar of each cell's own use
     double* sb;            // stencil adjoints [k][N + 2][S]
     double* grad;          // gradient planes [GS_COUNT][S], accumulated
