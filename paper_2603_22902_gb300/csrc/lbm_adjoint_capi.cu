@@ -157,7 +157,8 @@ extern "C" int lbm_adjoint_fl_loss(lbm_handle* h, const double* phi0, const doub
 
     // ---- forward: initial state, steps with a checkpoint every K ----
     cudaError_t e = dispatch(N, LBM_FP64, [&](auto n, auto pr) {
-        return launch_init<decltype(n)::value, decltype(pr)>(P, d_phi0, d_T0, d_ux0, d_uy0, h->pop[0], h->aux[0], st);
+        return launch_init<decltype(n)::value, decltype(pr)>(P, d_phi0, d_T0, d_ux0, d_uy0, h->pop[0], h->aux[0], h->sms,
+                                                             st);
     });
     if (e != cudaSuccess) return acuda(h, e, "init kernel");
     h->cur = 0;

@@ -392,7 +392,8 @@ int lbm_set_fields(lbm_handle* h, const double* phi, const double* T, const doub
     }
     h->cur = 0;
     cudaError_t e = dispatch(h->N, h->precision, [&](auto n, auto pr) {
-        return launch_init<decltype(n)::value, decltype(pr)>(h->P, dphi, dT, dux, duy, h->pop[0], h->aux[0], h->stream);
+        return launch_init<decltype(n)::value, decltype(pr)>(h->P, dphi, dT, dux, duy, h->pop[0], h->aux[0], h->sms,
+                                                             h->stream);
     });
     if (e != cudaSuccess) return cuda_fail(h, e, "init kernel");
     if (where == LBM_HOST) LBM_CUDA_TRY(h, cudaStreamSynchronize(h->stream));

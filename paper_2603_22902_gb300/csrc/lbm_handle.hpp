@@ -42,9 +42,9 @@ struct lbm_handle {
 };
 
 // Tile shape of the handle's one-launch step.
-inline int lbm_step_tile(const lbm_handle* h)
+inline lbm::StepTile lbm_step_tile(const lbm_handle* h)
 {
-    return h->tile_auto && h->precision == LBM_FP64 ? lbm::fp64_tile(h->nx, h->ny, h->sms) : h->tile;
+    return {h->tile_auto && h->precision == LBM_FP64 ? lbm::fp64_tile(h->nx, h->ny, h->sms) : h->tile, h->sms};
 }
 
 // The six tensor maps of the staged step (boxes A..F of lbm_staged.cuh) over a population

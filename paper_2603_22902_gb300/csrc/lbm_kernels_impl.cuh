@@ -38,7 +38,7 @@ static cudaError_t launch_overlapped(void (*kernel)(Params...), int blocks, int 
 
 template <int N, int TX, int TY, bool COLLIDE, class Pr>
 static cudaError_t launch_fused_t(const KParams& P, const void* pin, void* pout, const void* ain, void* aout,
-                                  ExportPtrs ex, cudaStream_t st, TileRows rows)
+                                  ExportPtrs ex, int sms, cudaStream_t st, TileRows rows)
 {
     using TA = typename Pr::TA;
     const int tiles = ((P.nx + TX - 1) / TX) * tile_rows_count((P.ny + TY - 1) / TY, rows);
@@ -47,10 +47,6 @@ static cudaError_t launch_fused_t(const KParams& P, const void* pin, void* pout,
         // one-warp tiles: the next launch's blocks crowd the SMs that have room first, and an FP64 step
         // is as long as its fullest SM's (Janus 300 x 150: 85 against 58 us), so launches with more
         // than a block to an SM do not overlap
-        int dev = 0, sms = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
         const bool team = fp64_ring_team(tiles, sms);
         const auto kernel = team ? fused_step_kernel<N, TX, TY, COLLIDE, Pr, true> : fused_step_kernel<N, TX, TY, COLLIDE, Pr>;
         const int threads = team ? 2 * TX * TY : TX * TY;
@@ -70,26 +66,26 @@ constexpr bool single_shape() { return std::is_same<Pr, PrecDF64>::value; }
 
 template <int N, bool COLLIDE, class Pr>
 static cudaError_t launch_fused(const KParams& P, const void* pin, void* pout, const void* ain, void* aout,
-                                ExportPtrs ex, int tile, cudaStream_t st, TileRows rows = TileRows{ROWS_ALL, 0, 0})
+                                ExportPtrs ex, StepTile tile, cudaStream_t st, TileRows rows = TileRows{ROWS_ALL, 0, 0})
 {
     if constexpr (single_shape<Pr>()) {
-        return launch_fused_t<N, 32, 8, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
+        return launch_fused_t<N, 32, 8, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, tile.sms, st, rows);
     } else {
-        switch (tile) {
-            case TILE_32x4: return launch_fused_t<N, 32, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
-            case TILE_64x4: return launch_fused_t<N, 64, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
-            case TILE_16x16: return launch_fused_t<N, 16, 16, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
+        switch (tile.id) {
+            case TILE_32x4: return launch_fused_t<N, 32, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, tile.sms, st, rows);
+            case TILE_64x4: return launch_fused_t<N, 64, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, tile.sms, st, rows);
+            case TILE_16x16: return launch_fused_t<N, 16, 16, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, tile.sms, st, rows);
             case TILE_8x4:
                 if constexpr (std::is_same<Pr, PrecFP64>::value)
-                    return launch_fused_t<N, 8, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
+                    return launch_fused_t<N, 8, 4, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, tile.sms, st, rows);
                 else return cudaErrorNotSupported;
-            default: return launch_fused_t<N, 32, 8, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, st, rows);
+            default: return launch_fused_t<N, 32, 8, COLLIDE, Pr>(P, pin, pout, ain, aout, ex, tile.sms, st, rows);
         }
     }
 }
 
 template <int N, class Pr>
-cudaError_t launch_step(const KParams& P, const void* pin, void* pout, const void* ain, void* aout, int tile,
+cudaError_t launch_step(const KParams& P, const void* pin, void* pout, const void* ain, void* aout, StepTile tile,
                         cudaStream_t st, TileRows rows)
 {
     return launch_fused<N, true, Pr>(P, pin, pout, ain, aout, ExportPtrs{}, tile, st, rows);
@@ -97,10 +93,10 @@ cudaError_t launch_step(const KParams& P, const void* pin, void* pout, const voi
 
 template <int N, class Pr>
 cudaError_t launch_export(const KParams& P, const void* pin, const void* ain, double* phi, double* T, double* H,
-                          double* fl, double* ux, double* uy, double* p, int tile, cudaStream_t st)
+                          double* fl, double* ux, double* uy, double* p, StepTile tile, cudaStream_t st)
 {
     return launch_fused<N, false, Pr>(P, pin, nullptr, ain, nullptr, ExportPtrs{phi, T, H, fl, ux, uy, p},
-                                      tile == TILE_8x4 ? TILE_8x4 : TILE_32x8, st);
+                                      StepTile{tile.id == TILE_8x4 ? TILE_8x4 : TILE_32x8, tile.sms}, st);
 }
 
 template <int N, class Pr>
@@ -125,11 +121,11 @@ cudaError_t launch_staged(const KParams& P, const StageMaps& maps, const void* p
 
 template <int N, class Pr>
 cudaError_t launch_init(const KParams& P, const double* phi, const double* T, const double* ux, const double* uy,
-                        void* pop, void* aux, cudaStream_t st)
+                        void* pop, void* aux, int sms, cudaStream_t st)
 {
-    // blocks of two warps where the lattice would leave SMs without one of eight (FP64, film
+    // blocks of two warps where the lattice would leave SMs without two of eight (FP64, film
     // 16x256: 16 blocks and 16 us against 64 blocks and 9 us)
-    const int nt = P.S < 256 * 304 ? 64 : 256;
+    const int nt = P.S < 2LL * 256 * sms ? 64 : 256;
     long long blocks = (P.S + nt - 1) / nt;
     if (blocks > 65535) blocks = 65535;
     init_kernel<N, Pr><<<(int)blocks, nt, 0, st>>>(P, phi, T, ux, uy, pop, (typename Pr::TA*)aux);
@@ -280,14 +276,14 @@ cudaError_t launch_adj_init(const KParams& P, const double* phi0, const double* 
                                             cudaStream_t);
 
 #define LBM_INSTANTIATE(N, PR)                                                                                      \
-    template cudaError_t launch_step<N, PR>(const KParams&, const void*, void*, const void*, void*, int,           \
+    template cudaError_t launch_step<N, PR>(const KParams&, const void*, void*, const void*, void*, StepTile,      \
                                             cudaStream_t, TileRows);                                                \
     template cudaError_t launch_staged<N, PR>(const KParams&, const StageMaps&, const void*, void*, const void*,   \
                                               void*, int*, cudaStream_t, TileRows);                                 \
     template cudaError_t launch_export<N, PR>(const KParams&, const void*, const void*, double*, double*, double*, \
-                                              double*, double*, double*, double*, int, cudaStream_t);               \
+                                              double*, double*, double*, double*, StepTile, cudaStream_t);          \
     template cudaError_t launch_init<N, PR>(const KParams&, const double*, const double*, const double*,           \
-                                            const double*, void*, void*, cudaStream_t);                             \
+                                            const double*, void*, void*, int, cudaStream_t);                        \
     template cudaError_t launch_diag<N, PR>(const KParams&, const void*, const void*, double*, double*, cudaStream_t, \
                                             long long, long long);                                                  \
     template cudaError_t launch_batch_persistent<N, PR>(const BatchTable&, int, int, int, cudaStream_t);            \

@@ -27,6 +27,11 @@ inline bool tile_dims(int id, int& tx, int& ty)
     }
 }
 
+// The tile shape of a handle's step launches, and the SMs of its device (the launchers' rules).
+struct StepTile {
+    int id, sms;
+};
+
 // Whether an FP64 step over `tiles` tiles of 256 cells (32x8, 64x4, 16x16), which `subtiles` tiles of
 // 8x4 cover as well, should use the latter.  The step is bound by the SM's 2-lane FP64 unit, which
 // a warp instruction holds for 16 cycles, so its time is the warp-passes on the fullest SM: a
@@ -61,14 +66,14 @@ inline int fp64_tile(int nx, int ny, int sms)
 }
 
 template <int N, class Pr>
-cudaError_t launch_step(const KParams& P, const void* pin, void* pout, const void* ain, void* aout, int tile,
+cudaError_t launch_step(const KParams& P, const void* pin, void* pout, const void* ain, void* aout, StepTile tile,
                         cudaStream_t st, TileRows rows = TileRows{ROWS_ALL, 0, 0});
 template <int N, class Pr>
 cudaError_t launch_export(const KParams& P, const void* pin, const void* ain, double* phi, double* T, double* H,
-                          double* fl, double* ux, double* uy, double* p, int tile, cudaStream_t st);
+                          double* fl, double* ux, double* uy, double* p, StepTile tile, cudaStream_t st);
 template <int N, class Pr>
 cudaError_t launch_init(const KParams& P, const double* phi, const double* T, const double* ux, const double* uy,
-                        void* pop, void* aux, cudaStream_t st);
+                        void* pop, void* aux, int sms, cudaStream_t st);
 // The step with its inputs staged by the TMA (lbm_staged.cuh): policies with 16-bit moving
 // populations, N = 2 or 3, one block per tile.  maps are the six tensor maps of the input set;
 // status receives 1 when an mbarrier wait gave up.  cudaErrorNotSupported for other policies.

@@ -151,7 +151,7 @@ bool message_rows(const lbm_handle* h, int side, int phase, bool pack, SlabRows&
 TileRows slab_rows(const lbm_handle* h, int part)
 {
     int tx = 32, ty = 8;
-    tile_dims(lbm_step_tile(h), tx, ty);
+    tile_dims(lbm_step_tile(h).id, tx, ty);
     const int tiles_y = (h->ny + ty - 1) / ty;
     const int lo = 1;                                              // rows >= ty, ring >= ty - 1 >= 2
     int hi = h->ny - 3 - ty >= 0 ? (h->ny - 3 - ty) / ty + 1 : 0;  // last row + 1 (ring) <= ny - 3
