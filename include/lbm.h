@@ -194,8 +194,10 @@ int lbm_debug_bounds(lbm_handle* h, long long* out3);
 /* Tile shape (bx, by) of the fused step kernel; 0, 0 restores the default (32x8).  The
  * shape must be one of the compiled variants, 32x8, 32x4, 64x4 or 16x16, and 32x8 for
  * an LBM_DF64 handle (LBM_EINVAL otherwise).  With no shape asked for, an LBM_FP64 handle
- * whose lattice fills the GPU badly with 32x8 tiles uses smaller ones.  Every operation is
- * rounded as written, so results do not depend on the shape. */
+ * whose lattice fills the GPU badly with 32x8 tiles uses smaller ones.  LBM_FP64, LBM_FP32
+ * and LBM_DF64 round every operation as written, so their results do not depend on the
+ * shape; those of 16-bit storage agree to rounding (their kernels leave the fusing of most
+ * products and sums to the compiler, for each shape on its own). */
 int lbm_set_tile(lbm_handle* h, int bx, int by);
 
 
@@ -352,11 +354,12 @@ typedef struct {
  * for nsteps steps, then evaluate L and its gradient by the hand-written reverse of
  * the fused step (discrete adjoint).
  * - The kinks of eq. H take the derivative of the branch the forward step took.
- * - The forward run keeps a copy of the state every checkpoint_every steps. The
- *   reverse sweep recomputes one segment at a time from its checkpoint, stores its
- *   states, and steps the adjoint back through them.
- * - Device memory: (nsteps / checkpoint_every + checkpoint_every + 2) states plus
- *   21 + 11 N planes of doubles, allocated for the duration of the call.
+ * - The forward run keeps a copy of the state every checkpoint_every steps, up to the last
+ *   segment, whose states it stores. The reverse sweep steps the adjoint back through
+ *   these; then it recomputes one segment at a time from its checkpoint and does the same.
+ * - Device memory: max(ceil(nsteps / K) - 1, 1) + K + 2 states, K = checkpoint_every (at
+ *   most max(nsteps, 1)), plus 44 + 12 N planes of doubles, allocated for the duration of
+ *   the call.
  * - FP64 handles only (LBM_EINVAL otherwise). fl_target and weight are [ny][nx] like
  *   the fields, in host or device memory per `where`.
  * - On return the handle holds the state after nsteps steps. Synchronises. */

@@ -40,7 +40,8 @@ struct StepTile {
 // more where every SM is full and win where the large ones leave SMs idle or unevenly filled.
 // Measured, us per step, 8x4 with one warp against 32x8, launches not overlapped (N = 2): 16 x 256 26.1 / 39.8, 128^2 28.6 / 38.0, 192^2
 // 41.1 / 38.6, 256^2 57.4 / 59.5, 384^2 117.5 / 114.5, 448^2 160 / 166, 512^2 201 / 193; the rule takes
-// the faster one at each of these, and for N = 3 and 4.
+// the faster one at each of these, and for N = 3 and 4.  It was fitted with one warp to a small tile: with
+// two (fp64_ring_team, up to four tiles to an SM) the small tiles are faster still where it takes them.
 inline bool fp64_small_tiles(long long tiles, long long subtiles, int sms)
 {
     return (subtiles + sms - 1) / sms * (6 + 1) < (tiles + sms - 1) / sms * (8 * 6 + 3);

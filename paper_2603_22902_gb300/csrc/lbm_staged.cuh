@@ -21,8 +21,9 @@
 // are either never read (beyond a wall or an outflow side: the ghost rule replaces them)
 // or, across a periodic side, read again from the cells they wrap to (wrap_item).  The
 // arithmetic is step_tile_l of the one-cell step with a loader that reads the stage, so
-// every cell is computed exactly as the one-cell step computes it (the two forms agree
-// bit for bit), and that code exists once in the kernel (a second copy for the tiles at
+// every cell is computed as the one-cell step computes it (the two forms agree bit for bit
+// for N = 2; for N = 3 one difference of products is fused in another way, gdiff_form in
+// lbm_cell16.cuh), and that code exists once in the kernel (a second copy for the tiles at
 // the sides, reading global memory, overflowed the instruction cache).  The tiles at the
 // sides run first (ring_first_tile).  Every wait on the mbarrier is bounded: a wait that
 // gives up sets a status word (reported as LBM_ETIMEOUT), waits (bounded) for the copies
