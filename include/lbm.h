@@ -204,9 +204,10 @@ int lbm_set_tile(lbm_handle* h, int bx, int by);
 /* Step with its inputs staged in shared memory by the tensor-memory accelerator: one
  * block per 32x8 tile, whose thread 0 copies the tile's populations and lagged values
  * (tile and ring) with six tensor copies; the tile is then computed from shared memory
- * (the arithmetic is that of lbm_step, cell by cell, bit for bit); positions beyond the
- * lattice are filled with zeros by the copies and, across a periodic side, read again
- * from the cells they wrap to.  A service of the library for LBM_FP16S and LBM_BF16S
+ * (the arithmetic is that of the one-launch form, cell by cell: bit for bit with N = 2;
+ * with N = 3 one difference of products is rounded in another order, so the forms agree
+ * to rounding); positions beyond the lattice are filled with zeros by the copies and,
+ * across a periodic side, read again from the cells they wrap to.  A service of the library for LBM_FP16S and LBM_BF16S
  * handles with N = 2 or 3, nx a multiple of 8 and the 32x8 tile, where it is on from
  * lbm_create (a handle whose tensor maps cannot be encoded runs the
  * one-launch form).  on = 0 returns to the one-launch form, on = 1 asks for the staged one

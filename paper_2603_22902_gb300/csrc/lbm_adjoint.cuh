@@ -24,7 +24,7 @@
 // coefficients alone, its moments come from mac_kernel's planes (so the cell kernel reads no
 // phase-field population), its quotients from one reciprocal, and the stencil adjoints of a cell away
 // from the sides go straight to their planes.  256 x 256, N = 4, us per launch, before and after:
-// mac 18 / 13, cell 306 / 208, moments 59 / 41.
+// mac 18 / 11, cell 306 / 206, moments 59 / 38.
 //
 // Parameter gradients accumulate per cell in FP64 planes (slot layout below) and are
 // reduced once at the end, in a fixed order.
@@ -264,7 +264,7 @@ __device__ __forceinline__ void stencil_source(const KParams& P, int x, int y, i
 // Threads of adj_cell_kernel: the cells at the sides first, in warps of their own, then the others.
 // A cell at a side takes several times the instructions of any other (push targets, wrapped and
 // ghost stencil points); in lattice order every row has two of them, and at 256 x 256 a quarter of
-// all warps ran both paths (272 us a launch; now 208).
+// all warps ran both paths (272 us a launch; now 206).
 __host__ __device__ inline long long adj_side_threads(int nx, int ny)
 {
     return ((2LL * nx + 2LL * (ny - 2)) + 31) / 32 * 32;

@@ -21,8 +21,9 @@ using init_t = typename std::conditional<std::is_same<R, float>::value, df64, d1
 // df64(double) (x rounded to FP32, and the rest rounded to FP32; of two equally near x the one
 // further from zero), put together with integer instructions.  The four FP64 instructions of
 // the conversion occupy a scheduler's share of the FP64 unit for 64 cycles each: the N + 3
-// inputs held that unit for 43 of the kernel's 78 us at 1024^2, N = 3, FP16 storage; now 64 us.  Only
-// values so small or so large that a part would leave FP32's normal range are converted there.
+// inputs held that unit for 43 of the kernel's 78 us at 1024^2, N = 3, FP16 storage, 64 us with
+// integers (89 since init_cell tests the roundings).  Only values so small or so large that a part
+// would leave FP32's normal range are converted there.
 template <class I>
 __device__ __forceinline__ I init_input(double x)
 {

@@ -320,7 +320,7 @@ int lbm_create(const lbm_grid* grid, int N, const lbm_phase* phases, const lbm_t
         return fail(nullptr, LBM_ENOMEM, "device allocation failed");
     }
     // the TMA-staged step is the default where it applies (it computes every cell as the
-    // one-launch form does, bit for bit)
+    // one-launch form does, bit for bit with N = 2 and to rounding with N = 3)
     if (enable_staging(h, false) != LBM_OK) cudaGetLastError();
     *out = h;
     return LBM_OK;

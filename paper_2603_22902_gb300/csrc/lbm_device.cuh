@@ -192,9 +192,9 @@ __host__ __device__ constexpr long long plane_cells_max(int elem_bytes) { return
 // Element c of plane `plane` of a block of planes.  The plane's address is the same for all
 // threads; only a 32-bit byte offset is each thread's own (plane_cells_max), so an access costs
 // few integer instructions.  With 64-bit indices per access, a third of the FP32
-// step's instructions were address arithmetic (N = 3: 690 of 1800 per cell, now 436; FP16 storage
-// N = 2: 280 of 1220, now 245); double words at 512^2 went from 65 to 60 us, FP16 storage from 18.7
-// to 17.2 us.
+// step's instructions were address arithmetic (N = 3: 690 of 1800 per cell, now 436); double words
+// at 512^2 went from 65 to 60 us.  (FP16 storage, N = 2, with the cell update of the other policies:
+// 280 of 1220 before and 245 after, 18.7 and 17.2 us.)
 template <class T>
 __device__ __forceinline__ T* plane_elem(T* base, const KParams& P, int plane, unsigned c)
 {

@@ -15,8 +15,8 @@ namespace lbm {
 
 // A launch that may start before the launch before it in the stream has ended: its kernel waits
 // (step_wait_previous) before it touches a population or lagged set.  Measured, us per step, against
-// plain launches: FP16 storage 512^2 15.0 / 16.6, 509 x 387 14.3 / 16.4, film 16 x 256 FP64 (one warp a tile) 23.8 / 26.3,
-// double words 512^2 60.2 / 61.7, 2048^2 FP16 storage no difference.  The batches, whose launches
+// plain launches: FP16 storage 512^2 16.1 / 18.4, 509 x 387 14.9 / 16.6, 2048^2 213.7 / 215.1, film 16 x 256 FP64 21.1 / 23.0,
+// double words 512^2 60.2 / 61.9.  The batches, whose launches
 // follow each other in a graph, gained nothing (32-case sweep 1.285 against 1.295 times the start) and
 // launch plainly.
 template <class... Params, class... Args>

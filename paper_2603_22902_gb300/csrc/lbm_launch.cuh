@@ -13,7 +13,7 @@
 namespace lbm {
 
 // Compiled tile shapes of the fused step kernel (TX x TY threads, one cell each).
-// TILE_8x4, one warp, is FP64's for small lattices and not among the shapes a caller can ask for.
+// TILE_8x4, one or two warps, is FP64's for small lattices and not among the shapes a caller can ask for.
 enum TileId { TILE_32x8 = 0, TILE_32x4 = 1, TILE_64x4 = 2, TILE_16x16 = 3, TILE_COUNT = 4, TILE_8x4 = 4 };
 inline bool tile_dims(int id, int& tx, int& ty)
 {
